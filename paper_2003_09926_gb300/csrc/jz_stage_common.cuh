@@ -114,10 +114,11 @@ __device__ __forceinline__ R eddy_nu(const KConst<R>& c, const R g[4][3], R Jn) 
     if (!(aa > tiny)) return R(0);
     return R(2.5) * c.cs2 * Fn<R>::jm23(Jn) * Fn<R>::sqrt_(Fn<R>::div(rmax(B, R(0)), aa));
   }
-  const R s12 = R(0.5) * (g[0][1] + g[1][0]), s13 = R(0.5) * (g[0][2] + g[2][0]);
-  const R s23 = R(0.5) * (g[1][2] + g[2][1]);
-  const R ss = g[0][0] * g[0][0] + g[1][1] * g[1][1] + g[2][2] * g[2][2] + R(2) * (s12 * s12 + s13 * s13 + s23 * s23);
-  return c.cs2 * Fn<R>::sqrt_(R(2) * ss) * Fn<R>::jm23(Jn);
+  // 2 S_ij S_ij with the off-diagonal sums 2 S_ab as they stand (factors of
+  // two are exact, so this rounds as the textbook form does)
+  const R s12 = g[0][1] + g[1][0], s13 = g[0][2] + g[2][0], s23 = g[1][2] + g[2][1];
+  const R ss2 = R(2) * (g[0][0] * g[0][0] + g[1][1] * g[1][1] + g[2][2] * g[2][2]) + (s12 * s12 + s13 * s13 + s23 * s23);
+  return c.cs2 * Fn<R>::sqrt_(ss2) * Fn<R>::jm23(Jn);
 }
 
 // ---------------------------------------------------------------------------

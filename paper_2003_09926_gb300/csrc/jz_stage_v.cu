@@ -20,21 +20,37 @@
 // constants plus once with the flags read at run time, and within a build
 // once per node role):
 //  - TMA stages the conserved variables of one plane (tile plus a two-node
-//    halo) into a planar buffer, and the metric fields of one plane (tile
-//    plus a one-node halo) into a second buffer; waits are bounded;
+//    halo) into a planar buffer, and the metric fields of two planes (tile
+//    plus a one-node halo) into two buffers; waits are bounded;
 //  - each staged plane is converted once into two rings of node records:
-//    conserved (rho, rho u, rho v, rho w | e) over four planes and primitive
-//    (u, v, w, T | p) over three, each a float4 plus a float, so that a
-//    node's stencil values arrive with two shared-memory loads;
+//    conserved (rho, rho u, rho v, rho w | e) over three planes and primitive
+//    (u, v, w, T | p) over two, each a float4 plus a float, so that a
+//    neighbour's stencil values arrive with two shared-memory loads;
 //  - one thread per node of the plus-shaped set (tile nodes plus the
 //    one-node i and j halo) forms G^k, the dissipation radius lambda~^k and
 //    the sensor nu^k of its node (tile threads in all three directions, halo
 //    threads in their own direction);
-//  - i and j face fluxes go through shared memory as float4 + float records,
-//    the k face flux of a column stays in its thread's registers;
+//  - i and j face fluxes go through shared memory as float4 + float records;
+//  - what only the thread itself reads again -- the records of its own column
+//    (planes t-1 .. t+3), the state of its k march, its own low face fluxes --
+//    is kept in tensor memory (tcgen05.ld / st), whose four lane quadrants
+//    together move four times the bytes per cycle of shared memory;
 //  - two block barriers per plane: node pass of plane t+1, k face, i/j
 //    residual and update of plane t | i/j face fluxes of plane t+1 and the
-//    conversion of the plane three ahead.
+//    conversion of the plane three ahead;
+//  - one loop body serves the whole chunk, the two planes that build up the
+//    k march included.
+//
+// What bounds it.  With the column in a shared-memory ring and a prologue of
+// its own, the kernel moved 7.8 shared-memory wavefronts per point through a
+// pipe 67% busy and stalled 0.9 cycles per instruction on instruction fetch
+// (103 KB of code for the three roles).  The column in tensor memory took the
+// wavefronts to 6.1, and the single loop body the code to 42 KB, the fetch
+// stalls to 0.2 and the issue rate from 53% to 65%: 0.360 to 0.301 ms per
+// stage on 256x192x192 (c1).  Tensor memory alone, with the old code size,
+// gained 1%: the fetch stalls rose by what the memory stalls fell.  Now issue
+// slots (65%) and the shared-memory pipe (64%) bind together, with the
+// barriers between.
 #include <cmath>
 #include <cstdint>
 
@@ -66,7 +82,6 @@ constexpr int NTILE = TI * TJ;                  // tile nodes
 constexpr int NJH = 2 * TI, NIH = 2 * TJ;       // j-halo (rows -1, TJ) and i-halo (columns -1, TI) nodes
 constexpr int NT = NTILE + NJH + NIH;           // threads (608 for 32 x 16 and 16 x 32)
 static_assert(NT % 32 == 0, "whole warps");
-constexpr int NCH = 3 * (NJH + NIH);            // plane elements converted by the halo threads
 constexpr int RW = TI + 4, RH = TJ + 4, PL = RW * RH;  // staged plane: tile + two-node halo (36 x 20)
 constexpr int MH = TJ + 2, MPL = RW * MH;        // metric box: rows -1 .. TJ, 36 columns
 // Warp layout of the tile threads.  A warp holds 32 nodes: a full row of a
@@ -80,10 +95,11 @@ constexpr bool ROWS4 = TI == 16 && TJ == 16;
 // i-halo warp fall on distinct banks (unpadded rows of 20 in the 16 x 16
 // build, for the warp layout above)
 constexpr int RR = ROWS4 ? RW : RW + 1, RPL = RR * RH;
-// ring depths (planes): conserved records 4 (the k face t + 1/2 reads
-// planes t-1 .. t+2), primitive records 3 (the node pass of plane t reads
-// planes t-1 .. t+1)
-constexpr int NSQ = 4, NSP = 3;
+// ring depths (planes): conserved records 3 (plane t + 1 for the faces, t + 2
+// for the own column's next record, t + 3 being converted), primitive
+// records 2 (the node pass of plane t + 1 reads planes t + 1 and, of its own
+// column, t + 2; t + 3 is converted after it)
+constexpr int NSQ = 3, NSP = 2;
 // node buffers: columns -1..TI / rows -1..TJ; face buffers: i faces 0..TI /
 // j faces 0..TJ.  The i-direction rows are padded (distinct banks for the
 // i-halo warp's column accesses; a stride of 20 in the 16 x 16 build).
@@ -93,7 +109,7 @@ constexpr size_t al(size_t x) { return (x + 127) / 128 * 128; }
 constexpr size_t RAW_B = al(4 * 5 * PL);
 constexpr size_t QV_B = al(16 * NSQ * RPL), QE_B = al(4 * NSQ * RPL);
 constexpr size_t PV_B = al(16 * NSP * RPL), PP_B = al(4 * NSP * RPL);
-constexpr size_t MET_B = al(4 * 10 * MPL);
+constexpr size_t MET_B = al(4 * 10 * MPL);       // one plane; two are staged
 constexpr int UPL = RW * TJ;                     // Q^(0) box: tile rows, 36 columns
 constexpr size_t Q0_B = al(4 * 5 * UPL);
 constexpr size_t GI4_B = al(16 * TJ * GIW), GI1_B = al(4 * TJ * GIW);
@@ -110,7 +126,7 @@ constexpr size_t O_QE = O_QV + QV_B;
 constexpr size_t O_PV = O_QE + QE_B;
 constexpr size_t O_PP = O_PV + PV_B;
 constexpr size_t O_MET = O_PP + PP_B;
-constexpr size_t O_Q0 = O_MET + MET_B;
+constexpr size_t O_Q0 = O_MET + 2 * MET_B;
 constexpr size_t O_GI4 = O_Q0 + Q0_B;
 constexpr size_t O_GI1 = O_GI4 + GI4_B;
 constexpr size_t O_GJ4 = O_GI1 + GI1_B;
@@ -122,6 +138,7 @@ constexpr size_t O_HI1 = O_HI4 + HI4_B;
 constexpr size_t O_HJ4 = O_HI1 + HI1_B;
 constexpr size_t O_HJ1 = O_HJ4 + HJ4_B;
 constexpr size_t O_BAR = O_HJ1 + HJ1_B;
+constexpr size_t O_TMEM = O_BAR + 64;  // tensor memory address (written by the allocation)
 constexpr size_t BYTES = O_BAR + 128;
 // during a chunk's prologue three more raw planes are staged over the node
 // and face buffers, which are not in use yet
@@ -134,8 +151,17 @@ static_assert(MINB == 1 || 2 * (BYTES + 128 + 1024) <= 228 * 1024, "two CTAs per
 constexpr uint32_t RAW_TX = 4 * 5 * PL;
 constexpr uint32_t MET_TX = 4 * 10 * MPL;
 constexpr uint32_t Q0_TX = 4 * 5 * UPL;
-// mbarriers: 0 raw buffer, 1..3 prologue staging, 4 metrics, 5 Q^(0)
-constexpr int B_RAW = 0, B_MET = 4, B_Q0 = 5, NBAR = 6;
+// mbarriers: 0 raw buffer, 1..3 prologue staging, 4, 5 metrics, 6 Q^(0)
+constexpr int B_RAW = 0, B_MET = 4, B_Q0 = 6, NBAR = 7;
+// Tensor memory as a per-thread scratchpad (32-bit columns of the thread's
+// own lane; the warps that share a lane quadrant take T_COLS columns each):
+// four records (primitive 5, conserved 5) of the thread's own column of
+// nodes, the state of the k march (G^k 5, low k face flux 5, lambda~, nu, J)
+// and the node's own low i and j face fluxes (10).
+constexpr int T_REC = 10, T_MARCH = 4 * T_REC, T_FACE = T_MARCH + 13, T_COLS = T_FACE + 10;
+constexpr int T_GROUPS = (NT / 32 + 3) / 4;
+constexpr int T_ALLOC = T_GROUPS * T_COLS <= 256 ? 256 : 512;  // columns per CTA
+static_assert(T_GROUPS * T_COLS <= T_ALLOC && MINB * T_ALLOC <= 512, "tensor memory");
 }  // namespace vr
 
 __device__ __forceinline__ void ld5(const float4* v4, const float* v1, int i, float q[5]) {
@@ -165,15 +191,81 @@ __device__ __forceinline__ bool wait_v(uint64_t* bar, uint32_t parity, long long
   return mbar_try_wait(bar, parity) || mbar_wait_bounded(bar, parity, limit);
 }
 
+// --- tensor memory (tcgen05.ld / st, 32 lanes x 32 bits) --------------------
+// Every lane of a warp reads and writes its own lane of the warp's quadrant,
+// so the columns are private to a thread.  Loads are asynchronous: issue
+// them, then tm_wait, then tie() every loaded array before its first use
+// (the empty asm makes the uses depend on a statement after the wait).
+__device__ __forceinline__ void tm_ld5(uint32_t a, float r[5]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]) : "r"(a));
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=f"(r[4]) : "r"(a + 4));
+}
+__device__ __forceinline__ void tm_ld8(uint32_t a, float r[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+               : "r"(a));
+}
+__device__ __forceinline__ void tm_ld10(uint32_t a, float r[10]) {
+  tm_ld8(a, r);
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=f"(r[8]), "=f"(r[9]) : "r"(a + 8));
+}
+__device__ __forceinline__ void tm_ld13(uint32_t a, float r[13]) {
+  tm_ld8(a, r);
+  tm_ld5(a + 8, r + 8);
+}
+__device__ __forceinline__ void tm_st5(uint32_t a, const float r[5]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(r[0]), "f"(r[1]),
+               "f"(r[2]), "f"(r[3]));
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(a + 4), "f"(r[4]));
+}
+__device__ __forceinline__ void tm_st8(uint32_t a, const float r[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(a), "f"(r[0]),
+               "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]));
+}
+__device__ __forceinline__ void tm_st10(uint32_t a, const float r[10]) {
+  tm_st8(a, r);
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(a + 8), "f"(r[8]), "f"(r[9]));
+}
+__device__ __forceinline__ void tm_st13(uint32_t a, const float r[13]) {
+  tm_st8(a, r);
+  tm_st5(a + 8, r + 8);
+}
+__device__ __forceinline__ void tm_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void tie(float (&r)[N]) {
+#pragma unroll
+  for (int v = 0; v < N; ++v) asm volatile("" : "+f"(r[v]));
+}
+// allocation by warp 0, published through shared memory; ends with a barrier
+__device__ __forceinline__ void tm_alloc(unsigned char* smem) {
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(smem + vr::O_TMEM)),
+                 "r"(vr::T_ALLOC)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void tm_free(unsigned char* smem) {
+  __syncthreads();  // every warp is past its last access
+  if (threadIdx.x < 32)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(
+                     *reinterpret_cast<volatile uint32_t*>(smem + vr::O_TMEM)),
+                 "r"(vr::T_ALLOC));
+}
+
 // Node quantities of node (x, y) of plane kk: G^k = E^k - F^k, lambda~^k,
-// nu^k.  Primitive records of the planes below / at / above in slots sM, sC,
-// sP; the conserved record of the plane in slot qC.  DIR = 0: all three
-// directions; DIR = 1 / 2 / 3: direction i / j / k only.
+// nu^k.  The node's own column comes in registers: primitive records of the
+// planes below / at / above (pm, pc, pp: u, v, w, T, p) and rho and e; its i
+// and j neighbours from the primitive ring slot sC of the plane.  DIR = 0:
+// all three directions; DIR = 1 / 2 / 3: direction i / j / k only.
 template <int DIR, int MD>
 __device__ __forceinline__ void node_v(const float4* __restrict__ PV, const float* __restrict__ PP,
-                                       const float4* __restrict__ QV, const float* __restrict__ QE,
-                                       const float* __restrict__ met, int sM, int sC, int sP, int qC, int x, int y,
-                                       const KConst<float>& c, float G[3][5], float lt[3], float nu[3], float& Jn) {
+                                       const float* __restrict__ met, int sC, const float pm5[5], const float pc5[5],
+                                       const float pp5[5], float rho, float e, int x, int y, const KConst<float>& c,
+                                       float G[3][5], float lt[3], float nu[3], float& Jn) {
   using namespace vr;
   const int o = (y + 2) * RR + x + 2;
   const int mo = (y + 1) * RW + x + 2;
@@ -182,11 +274,7 @@ __device__ __forceinline__ void node_v(const float4* __restrict__ PV, const floa
   for (int f = 0; f < 9; ++f) S[f] = met[f * MPL + mo];
   Jn = met[9 * MPL + mo];
   const float4* pc = PV + sC;
-  const float4 r0 = pc[o];
-  const float u = r0.x, v = r0.y, w = r0.z, T = r0.w;
-  const float p = PP[sC + o];
-  const float rho = QV[qC + o].x;
-  const float e = QE[qC + o];
+  const float u = pc5[0], v = pc5[1], w = pc5[2], T = pc5[3], p = pc5[4];
   constexpr int K0 = DIR == 0 ? 0 : DIR - 1;  // DIR 3: direction k only
   constexpr int K1 = DIR == 0 ? 3 : DIR;
 
@@ -198,7 +286,7 @@ __device__ __forceinline__ void node_v(const float4* __restrict__ PV, const floa
   if (ModelFlags<MD>::viscous(c)) {
     // Cartesian gradients of u, v, w, T: J/2 sum_k S^k_m (phi_+ - phi_-)
     const float4 a0 = pc[o + 1], b0 = pc[o - 1], a1 = pc[o + RR], b1 = pc[o - RR];
-    const float4 a2 = PV[sP + o], b2 = PV[sM + o];
+    const float4 a2 = make_float4(pp5[0], pp5[1], pp5[2], pp5[3]), b2 = make_float4(pm5[0], pm5[1], pm5[2], pm5[3]);
     const float hJ = 0.5f * Jn;
     float g[4][3];
 #if VR_PACKED_FACES
@@ -294,26 +382,28 @@ __device__ __forceinline__ void node_v(const float4* __restrict__ PV, const floa
     float pm, pp;
     if (k == 0) { pm = PP[sC + o - 1]; pp = PP[sC + o + 1]; }
     else if (k == 1) { pm = PP[sC + o - RR]; pp = PP[sC + o + RR]; }
-    else { pm = PP[sM + o]; pp = PP[sP + o]; }
+    else { pm = pm5[4]; pp = pp5[4]; }
     nu[k] = Fn<float>::div(fabsf(pp - 2.f * p + pm), pp + 2.f * p + pm);
   }
 }
 
-// dissipative face flux between nodes a and b of a line m, a, b, p:
-// h = (Ga + Gb)/2 - lam [e2 (qb - qa) - e4 (qp - 3 qb + 3 qa - qm)],
-// lam = (lt_a + lt_b)/2, e2 = k2 max(nu_a, nu_b), e4 = max(0, k4 - e2)
+// twice the dissipative face flux between nodes a and b of a line m, a, b, p:
+// 2h = Ga + Gb - 2 lam [e2 (qb - qa) - e4 (qp - 3 qb + 3 qa - qm)],
+// 2 lam = lt_a + lt_b, e2 = k2 max(nu_a, nu_b), e4 = max(0, k4 - e2); the
+// update takes half the time step instead (powers of two: the same rounding,
+// four operations fewer per face)
 __device__ __forceinline__ void face_v(const KConst<float>& c, float2 La, float2 Lb, const float Ga[5],
                                        const float Gb[5], const float qm[5], const float qa[5], const float qb[5],
                                        const float qp[5], float h[5]) {
-  const float lam = 0.5f * (La.x + Lb.x);
+  const float lam = La.x + Lb.x;
   const float e2 = c.k2 * fmaxf(La.y, Lb.y);
   const float e4 = fmaxf(0.f, c.k4 - e2);
   const float l2 = lam * e2, l4 = lam * e4;
 #if VR_PACKED_FACES
-  // h = (Ga + Gb)/2 - l2 d1 + l4 d3 on component pairs (0, 1) and (2, 3)
+  // 2h = (Ga + Gb) - l2 d1 + l4 d3 on component pairs (0, 1) and (2, 3)
   // with packed FP32x2 operations (each lane rounds as its scalar
   // counterpart), component 4 in scalar form
-  const float2 m1 = make_float2(-1.f, -1.f), m3 = make_float2(-3.f, -3.f), hf = make_float2(0.5f, 0.5f);
+  const float2 m1 = make_float2(-1.f, -1.f), m3 = make_float2(-3.f, -3.f);
   const float2 ml2 = make_float2(-l2, -l2), pl4 = make_float2(l4, l4);
 #pragma unroll
   for (int v = 0; v < 4; v += 2) {
@@ -321,7 +411,7 @@ __device__ __forceinline__ void face_v(const KConst<float>& c, float2 La, float2
     const float2 m = make_float2(qm[v], qm[v + 1]), p = make_float2(qp[v], qp[v + 1]);
     const float2 d1 = __ffma2_rn(a, m1, b);                       // qb - qa
     const float2 d3 = __ffma2_rn(d1, m3, __ffma2_rn(m, m1, p));  // (qp - qm) - 3 d1
-    const float2 g = __fmul2_rn(hf, __fadd2_rn(make_float2(Ga[v], Ga[v + 1]), make_float2(Gb[v], Gb[v + 1])));
+    const float2 g = __fadd2_rn(make_float2(Ga[v], Ga[v + 1]), make_float2(Gb[v], Gb[v + 1]));
     const float2 r = __ffma2_rn(pl4, d3, __ffma2_rn(ml2, d1, g));
     h[v] = r.x;
     h[v + 1] = r.y;
@@ -329,14 +419,14 @@ __device__ __forceinline__ void face_v(const KConst<float>& c, float2 La, float2
   {
     const float d1 = qb[4] - qa[4];
     const float d3 = (qp[4] - qm[4]) - 3.f * d1;
-    h[4] = fmaf(l4, d3, fmaf(-l2, d1, 0.5f * (Ga[4] + Gb[4])));
+    h[4] = fmaf(l4, d3, fmaf(-l2, d1, Ga[4] + Gb[4]));
   }
 #else
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     const float d1 = qb[v] - qa[v];
     const float d3 = (qp[v] - qm[v]) - 3.f * d1;
-    h[v] = 0.5f * (Ga[v] + Gb[v]) - (l2 * d1 - l4 * d3);
+    h[v] = (Ga[v] + Gb[v]) - (l2 * d1 - l4 * d3);
   }
 #endif
 }
@@ -374,13 +464,6 @@ struct Smem {
   }
 };
 
-// A thread's own node data of one plane, kept in registers from the node
-// pass to the face pass.
-struct Own {
-  float Gi[5], Gj[5];  // node fluxes G^i, G^j
-  float2 Li, Lj;       // (lambda~, nu) in i and j
-};
-
 // Node role of thread tid (warps hold one role each): 0 tile node, 2 j-halo
 // node, 1 i-halo node.
 __device__ __forceinline__ int role_of(int tid) {
@@ -406,7 +489,6 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
   const int i0 = bx * TI, j0 = by * TJ;
   const int t0 = L.lo[2] + bz * X.kc;
   const int t1 = min(t0 + X.kc, L.hi[2] + 1);
-  const int pbase = t0 - 2;  // first staged plane
   const uint32_t xtx = st.stall ? kStallBytes : 0u;
   const long long wlim = st.stall ? kStallLimit : kWaitLimit;
 
@@ -454,203 +536,111 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
 
-  // parities: the raw buffer takes plane t0-2, then t0+2, t0+3, ...; the
-  // metric buffer planes t0-1, t0, ...
-  auto raw_parity = [&](int p) { return (uint32_t)((p - t0 - 1) & 1); };
-  auto met_parity = [&](int p) { return (uint32_t)((p - t0 + 1) & 1); };
-  // thread 0's record of copies in flight: bit b of pend = barrier b has an
-  // unwaited copy, bit b of ppar = the parity of that copy's phase
+  // thread 0's record of its copies: bit b of pend = barrier b has had one,
+  // bit b of ppar = the parity of the last one's phase
   uint32_t pend = 0, ppar = 0;
+  // bookkeeping of a copy thread 0 is about to issue on barrier b
+  auto begin_copy = [&](int b, uint32_t parity, uint32_t bytes) {
+    pend |= 1u << b;
+    ppar = (ppar & ~(1u << b)) | (parity << b);
+    fence_async_shared();
+    mbar_expect_tx(&sm.bar[b], bytes + xtx);
+  };
   auto issue_raw = [&](int p, int b, float* dst, uint32_t parity) {
-    if (tid == 0) {
-      pend |= 1u << b;
-      ppar = (ppar & ~(1u << b)) | (parity << b);
-      fence_async_shared();
-      mbar_expect_tx(&sm.bar[b], RAW_TX + xtx);
+    if (ROLE == 0 && tid == 0) {
+      begin_copy(b, parity, RAW_TX);
       tma_load_4d(dst, &X.tmQ[st.qin], &sm.bar[b], i0, j0, p + NG, 0);
     }
   };
+  // the raw buffer takes planes t0+1, t0+2, ...; the two metric buffers
+  // planes t0-1, t0, t0+1, ... in turn
+  auto raw_parity = [&](int p) { return (uint32_t)((p - t0 - 1) & 1); };
+  auto met_sel = [&](int p) { return (p - t0 + 1) & 1; };
+  auto met_parity = [&](int p) { return (uint32_t)(((p - t0 + 1) >> 1) & 1); };
+  auto met_buf = [&](int p) { return reinterpret_cast<float*>(smem + O_MET + met_sel(p) * MET_B); };
   auto issue_met = [&](int p) {
-    if (tid == 0) {
-      pend |= 1u << B_MET;
-      ppar = (ppar & ~(1u << B_MET)) | ((uint32_t)((p - t0 + 1) & 1) << B_MET);
-      fence_async_shared();
-      mbar_expect_tx(&sm.bar[B_MET], MET_TX + xtx);
-      tma_load_4d(sm.met, &X.tmMv, &sm.bar[B_MET], i0, j0 + 1, p + NG, 0);
+    if (ROLE == 0 && tid == 0) {
+      const int b = B_MET + met_sel(p);
+      begin_copy(b, met_parity(p), MET_TX);
+      tma_load_4d(met_buf(p), &X.tmMv, &sm.bar[b], i0, j0 + 1, p + NG, 0);
     }
   };
   bool ok = true;
   auto wait = [&](int b, uint32_t parity, int p) {
-    const bool r = wait_v(&sm.bar[b], parity, wlim);
-    if (tid == 0) {
-      if (r) pend &= ~(1u << b);
-      else if (atomicCAS(X.err, 0, 1) == 0) {
-        int* info = X.err + 1;
-        info[0] = b; info[1] = (int)parity; info[2] = p; info[3] = bx; info[4] = by; info[5] = bz; info[6] = st.qin;
+    if (wait_v(&sm.bar[b], parity, wlim)) return;
+    ok = false;
+    if (ROLE == 0 && tid == 0 && atomicCAS(X.err, 0, 1) == 0) {
+      int* info = X.err + 1;
+      info[0] = b; info[1] = (int)parity; info[2] = p; info[3] = bx; info[4] = by; info[5] = bz; info[6] = st.qin;
+    }
+  };
+
+  // this thread's node in a ring plane, and its tensor-memory columns
+  const int oo = (ny + 2) * RR + nx + 2;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const uint32_t tm = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(smem + O_TMEM), 0) +
+                      ((uint32_t)(warp & 3) << 21) + (uint32_t)((warp >> 2) * T_COLS);
+
+  // Convert a staged plane (planar, in src) into the records of conserved
+  // slot sq and primitive slot sp: every thread its own node, whose record
+  // also goes to its tensor-memory record rec; halo threads the next node
+  // outwards too, and four of them the corners of the one-node halo (the
+  // outer corners are not read).
+  const int oraw = (ny + 2) * RW + nx + 2;
+  auto convert = [&](const float* src, int sq, int sp, int rec) {
+    int e = oraw, o = oo;
+    constexpr int NC = ROLE == 0 ? 1 : (ROLE == 2 ? 2 : 3);
+    bool on = true;
+#pragma unroll
+    for (int b = 0; b < NC; ++b) {
+      float r[10];
+      if (on) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) r[5 + v] = src[v * PL + e];
+        const float ri = Fn<float>::rcp(r[5]);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) r[m] = r[6 + m] * ri;
+        r[4] = c.gm1 * (r[9] - 0.5f * r[5] * (r[0] * r[0] + r[1] * r[1] + r[2] * r[2]));
+        r[3] = c.gamma * r[4] * ri;
+        st5(sm.QV + sq, sm.QE + sq, o, r + 5);
+        st5(sm.PV + sp, sm.PP + sp, o, r);
+      }
+      if (b == 0) {
+        __syncwarp();
+        tm_st10(tm + rec, r);
+      }
+      if (ROLE == 2) {
+        const int d = ny < 0 ? -1 : 1;
+        e += d * RW;
+        o += d * RR;
+      }
+      if (ROLE == 1) {
+        const int h = tid - NTILE - NJH;
+        if (b == 0) {
+          const int d = nx < 0 ? -1 : 1;
+          e += d;
+          o += d;
+        } else {
+          on = h < 4;
+          const int cx = (h & 1) ? TI + 2 : 1, cy = (h & 2) ? TJ + 2 : 1;
+          e = cy * RW + cx;
+          o = cy * RR + cx;
+        }
       }
     }
-    ok = ok && r;
-  };
-  // ring slots of plane p: conserved (p - pbase) mod 4, primitive mod 3
-  auto slot = [&](int p) { return ((p - pbase) & (NSQ - 1)) * RPL; };
-  auto pslot = [&](int p) { return ((p - pbase) % NSP) * RPL; };
-
-  // convert staged plane p (planar, in src) into the ring records: the
-  // conserved record (CQ) and / or the primitive record (CP)
-  auto convert_parts = [&](const float* src, int p, bool CQ, bool CP) {
-    float4* qv = sm.QV + slot(p);
-    float* qe = sm.QE + slot(p);
-    float4* pv = sm.PV + pslot(p);
-    float* pp = sm.PP + pslot(p);
-    // halo threads (lighter in the node pass) take three elements each, tile
-    // threads one or none
-    const int e0 = tid < NTILE ? NCH + tid : tid - NTILE;
-    const int e1 = tid < NTILE ? PL : NCH, es = tid < NTILE ? NTILE : NJH + NIH;
-    for (int e = e0; e < e1; e += es) {
-      const float q0 = src[e], q1 = src[PL + e], q2 = src[2 * PL + e], q3 = src[3 * PL + e], q4 = src[4 * PL + e];
-      const float ri = Fn<float>::rcp(q0);
-      const float u = q1 * ri, v = q2 * ri, w = q3 * ri;
-      const float pr = c.gm1 * (q4 - 0.5f * q0 * (u * u + v * v + w * w));
-      const int r = e + (RR - RW) * (e / RW);  // ring row (padded when RR > RW)
-      if (CQ) {
-        qv[r] = make_float4(q0, q1, q2, q3);
-        qe[r] = q4;
-      }
-      if (CP) {
-        pv[r] = make_float4(u, v, w, c.gamma * pr * ri);
-        pp[r] = pr;
-      }
-    }
-  };
-  auto convert = [&](const float* src, int p) { convert_parts(src, p, true, true); };
-
-  // node pass for plane kk: i/j node data to shared memory (for the
-  // neighbours' faces) and in registers (for this thread's own faces), k data
-  // in registers
-  auto node_pass = [&](int kk, Own& w, float G3[5], float& lt3, float& nu3, float& Jn) {
-    const int sM = pslot(kk - 1), sC = pslot(kk), sP = pslot(kk + 1), qC = slot(kk);
-    float G[3][5], lt[3], nu[3];
-    if (role == 0) {
-      node_v<0, MD>(sm.PV, sm.PP, sm.QV, sm.QE, sm.met, sM, sC, sP, qC, nx, ny, c, G, lt, nu, Jn);
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        w.Gi[v] = G[0][v];
-        w.Gj[v] = G[1][v];
-        G3[v] = G[2][v];
-      }
-      w.Li = make_float2(lt[0], nu[0]);
-      w.Lj = make_float2(lt[1], nu[1]);
-      st5(sm.Gi4, sm.Gi1, ny * GIW + nx + 1, w.Gi);
-      st5j(sm.Gj4, sm.Gj1, ny + 1, nx, w.Gj);
-      sm.Li[ny * GIW + nx + 1] = w.Li;
-      sm.Lj[(ny + 1) * TI + nx] = w.Lj;
-      lt3 = lt[2];
-      nu3 = nu[2];
-    } else if (role == 1) {
-      float Jh;
-      node_v<1, MD>(sm.PV, sm.PP, sm.QV, sm.QE, sm.met, sM, sC, sP, qC, nx, ny, c, G, lt, nu, Jh);
-#pragma unroll
-      for (int v = 0; v < 5; ++v) { w.Gi[v] = G[0][v]; w.Gj[v] = 0.f; }
-      w.Li = make_float2(lt[0], nu[0]);
-      w.Lj = make_float2(0.f, 0.f);
-      st5(sm.Gi4, sm.Gi1, ny * GIW + nx + 1, w.Gi);
-      sm.Li[ny * GIW + nx + 1] = w.Li;
-    } else {
-      float Jh;
-      node_v<2, MD>(sm.PV, sm.PP, sm.QV, sm.QE, sm.met, sM, sC, sP, qC, nx, ny, c, G, lt, nu, Jh);
-#pragma unroll
-      for (int v = 0; v < 5; ++v) { w.Gj[v] = G[1][v]; w.Gi[v] = 0.f; }
-      w.Lj = make_float2(lt[1], nu[1]);
-      w.Li = make_float2(0.f, 0.f);
-      st5j(sm.Gj4, sm.Gj1, ny + 1, nx, w.Gj);
-      sm.Lj[(ny + 1) * TI + nx] = w.Lj;
-    }
   };
 
-  // k data of plane kk only (tile threads), nothing written to shared memory
-  auto node_pass_k = [&](int kk, float G3[5], float& lt3, float& nu3, float& Jn) {
-    if (role != 0) return;
-    float G[3][5], lt[3], nu[3];
-    node_v<3, MD>(sm.PV, sm.PP, sm.QV, sm.QE, sm.met, pslot(kk - 1), pslot(kk), pslot(kk + 1), slot(kk), nx, ny, c, G,
-              lt, nu, Jn);
-#pragma unroll
-    for (int v = 0; v < 5; ++v) G3[v] = G[2][v];
-    lt3 = lt[2];
-    nu3 = nu[2];
-  };
-
-  // face fluxes of plane kk on the low side of this thread's node: i face
-  // between nx-1 and nx (tile nodes and the i-halo column TI), j face between
-  // ny-1 and ny (tile nodes and the j-halo row TJ).  The node's own G, (lt, nu)
-  // and conserved record come from registers; qo returns the record.
-  const bool do_i = role == 0 || (role == 1 && nx == TI);
-  const bool do_j = role == 0 || (role == 2 && ny == TJ);
-  const int oo = (ny + 2) * RR + nx + 2;  // this thread's node in a ring plane
-  auto face_pass = [&](int kk, const Own& w, float hi[5], float hj[5], float qo[5]) {
-    const float4* qv = sm.QV + slot(kk);
-    const float* qe = sm.QE + slot(kk);
-    if (do_i || do_j) ld5(qv, qe, oo, qo);
-    if (do_i) {
-      float Ga[5], q0[5], q1[5], q3[5];
-      ld5(sm.Gi4, sm.Gi1, ny * GIW + nx, Ga);
-      ld5(qv, qe, oo - 2, q0);
-      ld5(qv, qe, oo - 1, q1);
-      ld5(qv, qe, oo + 1, q3);
-      face_v(c, sm.Li[ny * GIW + nx], w.Li, Ga, w.Gi, q0, q1, qo, q3, hi);
-      st5(sm.Hi4, sm.Hi1, ny * HIW + nx, hi);
-    }
-    if (do_j) {
-      float Ga[5], q0[5], q1[5], q3[5];
-      ld5j(sm.Gj4, sm.Gj1, ny, nx, Ga);
-      ld5(qv, qe, oo - 2 * RR, q0);
-      ld5(qv, qe, oo - RR, q1);
-      ld5(qv, qe, oo + RR, q3);
-      face_v(c, sm.Lj[ny * TI + nx], w.Lj, Ga, w.Gj, q0, q1, qo, q3, hj);
-      st5j(sm.Hj4, sm.Hj1, ny, nx, hj);
-    }
-  };
-
-  // i/j residual of this thread's tile node from the four face fluxes
-  // around it (keeping the node's own faces in registers from the face
-  // phase through the next node pass would exceed the register budget)
-  auto rij = [&](float R[5]) {
-    float a[5], b[5], d[5], e[5];
-    ld5(sm.Hi4, sm.Hi1, ny * HIW + nx + 1, a);
-    ld5(sm.Hi4, sm.Hi1, ny * HIW + nx, d);
-    ld5j(sm.Hj4, sm.Hj1, ny + 1, nx, b);
-    ld5j(sm.Hj4, sm.Hj1, ny, nx, e);
-#pragma unroll
-    for (int v = 0; v < 5; ++v) R[v] = (a[v] - d[v]) + (b[v] - e[v]);
-  };
-
-  // k face flux between planes ka and ka+1 of this thread's column; q1 is
-  // the conserved record of plane ka+1 (already in registers)
-  auto kface = [&](int ka, const float Ga[5], const float Gb[5], float lta, float ltb, float nua, float nub,
-                   const float q1[5], float h[5]) {
-    float qm[5], qa[5], qp[5];
-    int s = slot(ka - 1);
-    ld5(sm.QV + s, sm.QE + s, oo, qm);
-    s = slot(ka);
-    ld5(sm.QV + s, sm.QE + s, oo, qa);
-    s = slot(ka + 2);
-    ld5(sm.QV + s, sm.QE + s, oo, qp);
-    face_v(c, make_float2(lta, nua), make_float2(ltb, nub), Ga, Gb, qm, qa, q1, qp, h);
-  };
-
-  const float adt = (float)(st.alpha * X.sc->dt);
+  const float hadt = 0.5f * (float)(st.alpha * X.sc->dt);  // half: the residual is formed of twice the face fluxes
   const long long npad = L.npad;
   float* const Qo = X.Q[st.qout];
   // Q^(0) of the plane being updated: for the first stage it is the stage
-  // input, still in the conserved ring; otherwise TMA stages it one plane
-  // ahead (tile rows, 36 columns from the aligned column i0-2)
-  const bool q0_ring = st.qin == 0;
+  // input, which the own column's records hold; otherwise TMA stages it one
+  // plane ahead (tile rows, 36 columns from the aligned column i0-2)
+  const bool q0_own = st.qin == 0;
   const float* q0buf = reinterpret_cast<const float*>(smem + O_Q0);
   auto issue_q0 = [&](int p) {
-    if (tid == 0 && !q0_ring) {
-      pend |= 1u << B_Q0;
-      ppar = (ppar & ~(1u << B_Q0)) | ((uint32_t)((p - t0) & 1) << B_Q0);
-      fence_async_shared();
-      mbar_expect_tx(&sm.bar[B_Q0], Q0_TX + xtx);
+    if (ROLE == 0 && tid == 0 && !q0_own) {
+      begin_copy(B_Q0, (uint32_t)((p - t0) & 1), Q0_TX);
       tma_load_4d(smem + O_Q0, &X.tmQ0u, &sm.bar[B_Q0], i0, j0 + 2, p + NG, 0);
     }
   };
@@ -658,110 +648,205 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
   float* scr[3] = {reinterpret_cast<float*>(smem + O_SCR), reinterpret_cast<float*>(smem + O_SCR + RAW_B),
                    reinterpret_cast<float*>(smem + O_SCR + 2 * RAW_B)};
 
-  // ---- prologue: planes t0-2 .. t0+1 staged at once and converted
-  issue_raw(t0 - 2, B_RAW, sm.raw, 0);
-  issue_raw(t0 - 1, 1, scr[0], 0);
-  issue_raw(t0, 2, scr[1], 0);
-  issue_raw(t0 + 1, 3, scr[2], 0);
+  // ---- prologue: planes t0-2 .. t0+1 and the metrics of t0-1, t0 staged at
+  // once; planes t0-1, t0 converted, the own column's records of t0-2 and
+  // t0-1 to tensor memory
+  issue_raw(t0 - 2, 1, scr[0], 0);
+  issue_raw(t0 - 1, 2, scr[1], 0);
+  issue_raw(t0, 3, scr[2], 0);
   issue_met(t0 - 1);
-  wait(B_RAW, 0, t0 - 2);
-  convert(sm.raw, t0 - 2);
-  wait(1, 0, t0 - 1);
-  convert(scr[0], t0 - 1);
-  wait(2, 0, t0);
-  convert(scr[1], t0);
-  wait(3, 0, t0 + 1);
-  // plane t0+1: conserved record now; its primitive slot still holds plane
-  // t0-2, which the node pass of plane t0-1 reads
-  convert_parts(scr[2], t0 + 1, true, false);
+  issue_raw(t0 + 1, B_RAW, sm.raw, 0);
+  issue_met(t0);
+#pragma unroll 1
+  for (int q = 0; q < 3; ++q) {  // primitive slots 1, 0, 1: plane t0's records replace t0-2's, which no other thread reads
+    wait(1 + q, 0, t0 - 2 + q);
+    convert(scr[0] + q * (RAW_B / 4), q * RPL, ((q + 1) & 1) * RPL, q * T_REC);
+  }
+  __syncwarp();
+  tm_wait_st();
   if (__syncthreads_or(!ok)) goto fail;
-  issue_raw(t0 + 2, B_RAW, sm.raw, raw_parity(t0 + 2));
 
   {
-    float G3m[5], lt3m = 0.f, nu3m = 0.f, Jm = 0.f;
-    float G3c[5], lt3c = 0.f, nu3c = 0.f, Jc = 0.f;
-    float hprev[5];
-    Own w;
-    // node pass of plane t0-1 (its k data only), of plane t0, the k face
-    // t0 - 1/2, the i/j faces of plane t0 and the conversion of plane t0+2
-    wait(B_MET, met_parity(t0 - 1), t0 - 1);
-    node_pass_k(t0 - 1, G3m, lt3m, nu3m, Jm);
-    if (__syncthreads_or(!ok)) goto fail;
-    issue_met(t0);
-    convert_parts(scr[2], t0 + 1, false, true);  // scr[2] is overwritten by the node pass below
-    if (__syncthreads_or(!ok)) goto fail;
-    wait(B_MET, met_parity(t0), t0);
-    node_pass(t0, w, G3c, lt3c, nu3c, Jc);
-    if (role == 0) {
-      float q1[5];
-      const int s = slot(t0);
-      ld5(sm.QV + s, sm.QE + s, oo, q1);
-      kface(t0 - 1, G3m, G3c, lt3m, lt3c, nu3m, nu3c, q1, hprev);
-    }
-    if (__syncthreads_or(!ok)) goto fail;
-    issue_met(t0 + 1);
-    issue_q0(t0);
-    {
-      float hi[5], hj[5], qo[5];
-      face_pass(t0, w, hi, hj, qo);
-    }
-    // ring slot of plane t0-2 is free: its last readers were the k face above
-    wait(B_RAW, raw_parity(t0 + 2), t0 + 2);
-    convert(sm.raw, t0 + 2);
-    if (__syncthreads_or(!ok)) goto fail;
-    if (t0 + 3 <= t1 + 1) issue_raw(t0 + 3, B_RAW, sm.raw, raw_parity(t0 + 3));
+    // the node's own face data, from the node pass to the face pass
+    float Gi[5], Gj[5];
+    float2 Li, Lj;
+    const bool do_i = role == 0 || (role == 1 && nx == TI);
+    const bool do_j = role == 0 || (role == 2 && ny == TJ);
 
-    // ---- march in k: iteration t writes plane t.  Phase 1: node pass of
-    // plane t+1, k face t + 1/2, i/j residual of plane t (faces from phase 2
-    // of the previous iteration) and the update of plane t.  Phase 2: i/j
-    // faces of plane t+1 and the conversion of plane t+3 (into the ring slot
-    // of plane t-1, whose last reader was the k face of phase 1).
-    for (int t = t0; t < t1; ++t) {
+    // ---- march in k: iteration t writes plane t (from t0 on; the two before
+    // it only build up the k march).  Phase 1: node pass of plane t+1, k face
+    // t + 1/2, i/j residual of plane t (faces from phase 2 of the previous
+    // iteration) and the update of plane t.  Phase 2: i/j faces of plane t+1
+    // and the conversion of plane t+3.  r0, r1, r2: conserved ring slots of
+    // planes t, t+1, t+2 (t+3 takes t's slot); k0: tensor-memory record of
+    // plane t (of four in turn).
+    int r0 = 0, r1 = RPL, r2 = 2 * RPL, k0 = 0;
+#pragma unroll 1
+    for (int t = t0 - 2; t < t1; ++t) {
+      const bool live = t + 1 >= t0 && t + 1 < t1;  // plane t+1 is updated: its faces are needed
+      const int sp1 = ((t - t0) & 1) * RPL;  // primitive slot of plane t+1
+      const int k1 = (k0 + 1) & 3, k2 = (k0 + 2) & 3, k3 = (k0 + 3) & 3;
+      float qb[5];  // own conserved record of plane t+1
       float G3n[5], lt3n = 0.f, nu3n = 0.f, Jn = 0.f;
-      wait(B_MET, met_parity(t + 1), t + 1);
-      node_pass(t + 1, w, G3n, lt3n, nu3n, Jn);
-      if (!q0_ring) wait(B_Q0, (uint32_t)((t - t0) & 1), t);
-      if (role == 0) {
-        float q1[5], hk[5], R[5];
-        const int s = slot(t + 1);
-        ld5(sm.QV + s, sm.QE + s, oo, q1);
-        kface(t, G3c, G3n, lt3c, lt3n, nu3c, nu3n, q1, hk);
-        rij(R);
-        if (own) {
+      wait(B_MET + met_sel(t + 1), met_parity(t + 1), t + 1);
+      __syncwarp();
+      {
+        float pb[5], pt[5], pn[5];
+        tm_ld5(tm + k0 * T_REC, pb);
+        tm_ld5(tm + k1 * T_REC, pt);
+        tm_ld5(tm + k1 * T_REC + 5, qb);
+        tm_ld5(tm + k2 * T_REC, pn);
+        tm_wait_ld();
+        tie(pb);
+        tie(pt);
+        tie(qb);
+        tie(pn);
+        const float* met = met_buf(t + 1);
+        float G[3][5], lt[3], nu[3];
+        if constexpr (ROLE == 0) {
+          node_v<0, MD>(sm.PV, sm.PP, met, sp1, pb, pt, pn, qb[0], qb[4], nx, ny, c, G, lt, nu, Jn);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) {
+            Gi[v] = G[0][v];
+            Gj[v] = G[1][v];
+            G3n[v] = G[2][v];
+          }
+          lt3n = lt[2];
+          nu3n = nu[2];
+        } else if (live) {
+          node_v<ROLE, MD>(sm.PV, sm.PP, met, sp1, pb, pt, pn, qb[0], qb[4], nx, ny, c, G, lt, nu, Jn);
+#pragma unroll
+          for (int v = 0; v < 5; ++v) {
+            if (ROLE == 1) Gi[v] = G[0][v];
+            else Gj[v] = G[1][v];
+          }
+        }
+        if (ROLE == 0 || live) {
+          if (ROLE != 2) {
+            Li = make_float2(lt[0], nu[0]);
+            st5(sm.Gi4, sm.Gi1, ny * GIW + nx + 1, Gi);
+            sm.Li[ny * GIW + nx + 1] = Li;
+          }
+          if (ROLE != 1) {
+            Lj = make_float2(lt[1], nu[1]);
+            st5j(sm.Gj4, sm.Gj1, ny + 1, nx, Gj);
+            sm.Lj[(ny + 1) * TI + nx] = Lj;
+          }
+        }
+      }
+      if (!q0_own && t >= t0) wait(B_Q0, (uint32_t)((t - t0) & 1), t);
+      if constexpr (ROLE == 0) {
+        float mv[13], hl[10], qc[5], qd[5], qp[5], hk[5];
+        __syncwarp();
+        tm_ld13(tm + T_MARCH, mv);
+        tm_ld5(tm + k3 * T_REC + 5, qc);  // plane t-1
+        tm_ld5(tm + k0 * T_REC + 5, qd);
+        tm_ld5(tm + k2 * T_REC + 5, qp);
+        tm_wait_ld();
+        tie(mv);
+        tie(qc);
+        tie(qd);
+        tie(qp);
+        tm_ld10(tm + T_FACE, hl);
+        face_v(c, make_float2(mv[10], mv[11]), make_float2(lt3n, nu3n), mv, G3n, qc, qd, qb, qp, hk);
+        {
+          float nv[13];
+#pragma unroll
+          for (int v = 0; v < 5; ++v) {
+            nv[v] = G3n[v];
+            nv[5 + v] = hk[v];
+          }
+          nv[10] = lt3n;
+          nv[11] = nu3n;
+          nv[12] = Jn;
+          tm_st13(tm + T_MARCH, nv);
+        }
+        // i/j residual from the four face fluxes around the node: its own low
+        // ones from tensor memory, the high ones of its neighbours' threads
+        float hi[5], hj[5];
+        ld5(sm.Hi4, sm.Hi1, ny * HIW + nx + 1, hi);
+        ld5j(sm.Hj4, sm.Hj1, ny + 1, nx, hj);
+        tm_wait_ld();
+        tie(hl);
+        if (own && t >= t0) {
           float q0[5];
-          if (q0_ring) {
-            const int s0 = slot(t);
-            ld5(sm.QV + s0, sm.QE + s0, oo, q0);
+          if (q0_own) {
+#pragma unroll
+            for (int v = 0; v < 5; ++v) q0[v] = qd[v];
           } else {
 #pragma unroll
             for (int v = 0; v < 5; ++v) q0[v] = q0buf[v * UPL + ny * RW + nx + 2];
           }
-          const long long n = n_t0 + (long long)(t - t0) * L.plane;
+          float* const dst = Qo + n_t0 + (long long)(t - t0) * L.plane;
+          const float aj = -(hadt * mv[12]);
+          float qn[5];
+          const float2 m1 = make_float2(-1.f, -1.f), aj2 = make_float2(aj, aj);
 #pragma unroll
-          for (int v = 0; v < 5; ++v) Qo[v * npad + n] = q0[v] - adt * Jc * (R[v] + (hk[v] - hprev[v]));
-        }
+          for (int v = 0; v < 4; v += 2) {  // packed pairs, each lane rounding as its scalar counterpart
+            const float2 di = __ffma2_rn(make_float2(hl[v], hl[v + 1]), m1, make_float2(hi[v], hi[v + 1]));
+            const float2 dj = __ffma2_rn(make_float2(hl[5 + v], hl[6 + v]), m1, make_float2(hj[v], hj[v + 1]));
+            const float2 dk = __ffma2_rn(make_float2(mv[5 + v], mv[6 + v]), m1, make_float2(hk[v], hk[v + 1]));
+            const float2 r = __ffma2_rn(aj2, __fadd2_rn(__fadd2_rn(di, dj), dk), make_float2(q0[v], q0[v + 1]));
+            qn[v] = r.x;
+            qn[v + 1] = r.y;
+          }
+          qn[4] = fmaf(aj, ((hi[4] - hl[4]) + (hj[4] - hl[9])) + (hk[4] - mv[9]), q0[4]);
 #pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          G3c[v] = G3n[v];
-          hprev[v] = hk[v];
+          for (int v = 0; v < 5; ++v) dst[v * npad] = qn[v];
         }
-        lt3c = lt3n;
-        nu3c = nu3n;
-        Jc = Jn;
       }
+      __syncwarp();
+      tm_wait_st();
       if (__syncthreads_or(!ok)) goto fail;
-      if (t + 2 <= t1) issue_met(t + 2);
-      if (t + 1 < t1) issue_q0(t + 1);
-      if (t + 1 < t1) {
-        float hi[5], hj[5], qo[5];
-        face_pass(t + 1, w, hi, hj, qo);
+      if (t + 3 <= t1) issue_met(t + 3);
+      // face fluxes (twice) of plane t+1 on the low side of this thread's
+      // node: i face between nx-1 and nx (tile nodes and the i-halo column
+      // TI), j face between ny-1 and ny (tile nodes and the j-halo row TJ).
+      // A tile node keeps its two faces in tensor memory for its residual.
+      if (live) {
+        issue_q0(t + 1);
+        const float4* qv = sm.QV + r1;
+        const float* qe = sm.QE + r1;
+        float qo[5], hij[10];
+        __syncwarp();
+        tm_ld5(tm + k1 * T_REC + 5, qo);
+        tm_wait_ld();
+        tie(qo);
+        if (do_i) {
+          float Ga[5], qm[5], qa[5], qp[5];
+          ld5(sm.Gi4, sm.Gi1, ny * GIW + nx, Ga);
+          ld5(qv, qe, oo - 2, qm);
+          ld5(qv, qe, oo - 1, qa);
+          ld5(qv, qe, oo + 1, qp);
+          face_v(c, sm.Li[ny * GIW + nx], Li, Ga, Gi, qm, qa, qo, qp, hij);
+          st5(sm.Hi4, sm.Hi1, ny * HIW + nx, hij);
+        }
+        if (do_j) {
+          float Ga[5], qm[5], qa[5], qp[5];
+          ld5j(sm.Gj4, sm.Gj1, ny, nx, Ga);
+          ld5(qv, qe, oo - 2 * RR, qm);
+          ld5(qv, qe, oo - RR, qa);
+          ld5(qv, qe, oo + RR, qp);
+          face_v(c, sm.Lj[ny * TI + nx], Lj, Ga, Gj, qm, qa, qo, qp, hij + 5);
+          st5j(sm.Hj4, sm.Hj1, ny, nx, hij + 5);
+        }
+        if constexpr (ROLE == 0) {
+          tm_st10(tm + T_FACE, hij);
+        }
       }
       if (t + 3 <= t1 + 1) {
         wait(B_RAW, raw_parity(t + 3), t + 3);
-        convert(sm.raw, t + 3);
+        convert(sm.raw, r0, sp1, k3 * T_REC);
+        __syncwarp();
+        tm_wait_st();
       }
       if (__syncthreads_or(!ok)) goto fail;
       if (t + 4 <= t1 + 1) issue_raw(t + 4, B_RAW, sm.raw, raw_parity(t + 4));
+      const int r = r0;
+      r0 = r1;
+      r1 = r2;
+      r2 = r;
+      k0 = k1;
     }
   }
   return true;
@@ -784,11 +869,13 @@ template <int MD>
 __global__ void __launch_bounds__(vr::NT, vr::MINB)
     k_stage_v(const __grid_constant__ StageCtx<float, float> X, const StageSel st) {
   extern __shared__ __align__(128) unsigned char smem[];
+  tm_alloc(smem);
   switch (role_of(threadIdx.x)) {
     case 0: item_v<MD, 0>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
     case 2: item_v<MD, 2>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
     default: item_v<MD, 1>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
   }
+  tm_free(smem);
 }
 
 template <int MD>
@@ -798,6 +885,7 @@ __global__ void __launch_bounds__(vr::NT, vr::MINB)
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int next;
   bool first = true;
+  tm_alloc(smem);
   for (;;) {
     if (threadIdx.x == 0) next = (int)atomicAdd(queue, 1u);
     __syncthreads();
@@ -814,6 +902,7 @@ __global__ void __launch_bounds__(vr::NT, vr::MINB)
     if (!ok) break;
     first = false;
   }
+  tm_free(smem);
 }
 
 template <int MD>
