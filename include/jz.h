@@ -326,8 +326,9 @@ int jz_state_upload(jz_grid* g, const double* host, size_t n);
  * CTAs take (grid, tile, k-chunk) work items from a device queue, largest
  * first, plus one batched boundary fill (preceded by the centreline means
  * when a grid is cylindrical); per step one batched time-step reduction.  The batch borrows the grids (one precision mode, flow
- * parameters set; they must outlive the batch and keep the k-chunk length
- * they had at jz_batch_create) and a caller-owned, 256-byte aligned device
+ * parameters set; they must outlive the batch; a k-chunk length set with
+ * jz_set_tiling is kept, the others are chosen for the whole batch) and a
+ * caller-owned, 256-byte aligned device
  * buffer of jz_batch_bytes bytes for its tables; work goes to `stream`
  * (the grids' own streams are not used, so order them against it).  Every
  * grid keeps its own CFL time step on the device, and its state is bitwise

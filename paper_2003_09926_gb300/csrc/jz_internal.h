@@ -27,6 +27,7 @@ struct GridDev {
   double* axis;        // centreline values of a cylindrical grid, [5][ni] FP64 (set per boundary pass)
   FlowC F;
   int kc;              // planes per CTA chunk of the stage kernel
+  int kc_set;          // kc was set by the caller (a batch then keeps it)
   int goff[3], gn[3];  // global index of local node 0 and global node counts (blocks; else 0 and n)
   int variant;         // stage kernel of P32: 0 scalar records, 2 vector records
   int vti, vtj;        // tile shape of the vector-record kernel (32 x 16, 16 x 32 or 16 x 16)
