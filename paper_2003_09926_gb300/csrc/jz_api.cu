@@ -449,7 +449,7 @@ int create_grid(const jz_grid_desc* desc, const int* o0, const int* o1, void* de
   d.partial = (double*)(g->base + cv.off_partial);
   d.inflow = (double*)(g->base + cv.off_inflow);
   d.axis = (double*)(g->base + cv.off_axis);
-  d.variant = d.prec == JZ_P32 ? 2 : 0;  // P32: the vector-record kernel (fastest measured)
+  d.variant = (d.prec == JZ_P32 || d.prec == JZ_P32_S64) ? 2 : 0;  // the vector-record kernel where it is built
   d.vti = 16;  // two CTAs per SM; as fast as 32 x 16 on 256x192x192, faster on small grids
   d.vtj = 16;
   d.kc = default_kc(cv.L, grid_tiling(d), grid_ctas_per_sm(d));
@@ -772,6 +772,7 @@ int jz_set_stage_variant(jz_grid* g, int variant) {
   if (int rc = check_grid(g, false)) return rc;
   if (variant != 0 && variant != 2) return fail(JZ_EINVAL, "stage variant must be 0 or 2");
   if (variant != 0 && g->dev.prec != JZ_P32) return fail(JZ_EINVAL, "stage variant 2 is FP32 (JZ_P32) only");
+  if (g->dev.prec != JZ_P32) return JZ_OK;  // one kernel only
   g->dev.variant = variant;
   drop_graph(g);
   return build_maps(g->dev);  // the two kernels may stage different tiles

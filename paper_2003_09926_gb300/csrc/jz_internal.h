@@ -29,7 +29,7 @@ struct GridDev {
   int kc;              // planes per CTA chunk of the stage kernel
   int kc_set;          // kc was set by the caller (a batch then keeps it)
   int goff[3], gn[3];  // global index of local node 0 and global node counts (blocks; else 0 and n)
-  int variant;         // stage kernel of P32: 0 scalar records, 2 vector records
+  int variant;         // stage kernel: 2 vector records (P32 by default, P32_S64), 0 scalar records
   int vti, vtj;        // tile shape of the vector-record kernel (32 x 16, 16 x 32 or 16 x 16)
   int stall_test;      // test only: the stage kernels' copies wait for bytes that nothing delivers
   int step_diag;       // each step's time-step reduction also forms the diagnostics of the state it reads
@@ -119,7 +119,7 @@ StageTiling stage_tiling(int prec);
 // the tile of the kernel a grid runs: its chosen shape for the FP32
 // vector-record kernel, else the fixed tile of its precision mode
 inline StageTiling grid_tiling(const GridDev& g) {
-  return (g.prec == JZ_P32 && g.variant == 2) ? StageTiling{g.vti, g.vtj} : stage_tiling(g.prec);
+  return g.variant == 2 ? StageTiling{g.vti, g.vtj} : stage_tiling(g.prec);
 }
 int stage_ctas_per_sm(int prec);
 // resident CTAs per SM of the stage kernel a grid runs

@@ -225,11 +225,7 @@ __device__ __forceinline__ void face5(const R* ring, const int so[4], const int 
 // One work item: the tile (bx, by) and k-chunk bz of grid X for stage st.
 // ph[] counts completed phases of the three mbarriers (identical in every
 // thread); issued[] / waited[] are kept by thread 0 for the timeout path.
-// S64: the state between time steps is FP64 (X.Q0d, interior nodes): the
-// update adds the FP32 increment to it in FP64, stages 1-4 round their
-// output to FP32 (it feeds only the FP32 flux evaluation), and stage 5 writes
-// both the FP64 state and its FP32 copy (the next step's flux input).
-template <typename R, typename MT, int TI, int TJ, bool S64, int MD>
+template <typename R, typename MT, int TI, int TJ, int MD>
 __device__ __forceinline__ void stage_item(const StageCtx<R, MT>& X, const StageSel& st, int bx, int by, int bz,
                                            unsigned char* smem, uint32_t ph[3], int issued[3], int waited[3],
                                            bool& failed) {
@@ -467,17 +463,11 @@ __device__ __forceinline__ void stage_item(const StageCtx<R, MT>& X, const Stage
   // ---- march in k
   for (int t = t0; t < t1 && !failed; ++t) {
     R q0[5];
-    double q0d[5];
     long long n = 0;
     if (own) {
       n = L.at(gi, gj, t);
-      if constexpr (S64) {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) q0d[v] = X.Q0d[v * npad + n];
-      } else {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) q0[v] = X.Q[0][v * npad + n];
-      }
+      for (int v = 0; v < 5; ++v) q0[v] = X.Q[0][v * npad + n];
     }
     // the barrier inside fetch_plane also orders the previous iteration's
     // reads of ring slot t-2 and of the face buffers before they are rewritten
@@ -492,17 +482,8 @@ __device__ __forceinline__ void stage_item(const StageCtx<R, MT>& X, const Stage
       R hk[5];
       kface(t, G3c, G3n, lt3c, lt3n, nu3c, nu3n, hk);
       if (own) {
-        if constexpr (S64) {
 #pragma unroll
-          for (int v = 0; v < 5; ++v) {
-            const double qn = q0d[v] - (double)(adt * Jc * (Rc[v] + (hk[v] - hprev[v])));
-            Qo[v * npad + n] = (R)qn;
-            if (st.qout == 0) X.Q0d[v * npad + n] = qn;
-          }
-        } else {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) Qo[v * npad + n] = q0[v] - adt * Jc * (Rc[v] + (hk[v] - hprev[v]));
-        }
+        for (int v = 0; v < 5; ++v) Qo[v * npad + n] = q0[v] - adt * Jc * (Rc[v] + (hk[v] - hprev[v]));
       }
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
@@ -520,7 +501,7 @@ __device__ __forceinline__ void stage_item(const StageCtx<R, MT>& X, const Stage
 
 // One grid: one CTA per (tile, k-chunk).  MD: the flow model (constant
 // flags, or read at run time).
-template <typename R, typename MT, int TI, int TJ, bool S64, int MD>
+template <typename R, typename MT, int TI, int TJ, int MD>
 __global__ void __launch_bounds__(Cfg<R, MT, TI, TJ>::NT, Cfg<R, MT, TI, TJ>::MINB)
     k_stage(const __grid_constant__ StageCtx<R, MT> X, const StageSel st) {
   using C = Cfg<R, MT, TI, TJ>;
@@ -530,7 +511,7 @@ __global__ void __launch_bounds__(Cfg<R, MT, TI, TJ>::NT, Cfg<R, MT, TI, TJ>::MI
   uint32_t ph[3] = {0, 0, 0};
   int issued[3] = {0, 0, 0}, waited[3] = {0, 0, 0};
   bool failed = false;
-  stage_item<R, MT, TI, TJ, S64, MD>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, ph, issued, waited, failed);
+  stage_item<R, MT, TI, TJ, MD>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, ph, issued, waited, failed);
   if (failed) drain_after_timeout(bar, X.err, issued, waited, st.stall ? kStallBytes : 0u);
 }
 
@@ -540,7 +521,7 @@ __global__ void __launch_bounds__(Cfg<R, MT, TI, TJ>::NT, Cfg<R, MT, TI, TJ>::MI
 // kMixedModels: each work item in the build of its own grid's model, as
 // when the grid is stepped alone.
 constexpr int kMixedModels = -1;
-template <typename R, typename MT, int TI, int TJ, bool S64, int MD>
+template <typename R, typename MT, int TI, int TJ, int MD>
 __global__ void __launch_bounds__(Cfg<R, MT, TI, TJ>::NT, Cfg<R, MT, TI, TJ>::MINB)
     k_stage_batch(const StageCtx<R, MT>* __restrict__ ctx, const int4* __restrict__ items, int nitems,
                   unsigned int* queue, const StageSel st) {
@@ -562,9 +543,9 @@ __global__ void __launch_bounds__(Cfg<R, MT, TI, TJ>::NT, Cfg<R, MT, TI, TJ>::MI
     const int4 w = items[it];
     gsel = w.x;
     if (MD == kModelSmagorinsky || (MD == kMixedModels && flow_model(ctx[w.x].k) == kModelSmagorinsky))
-      stage_item<R, MT, TI, TJ, S64, kModelSmagorinsky>(ctx[w.x], st, w.y, w.z, w.w, smem, ph, issued, waited, failed);
+      stage_item<R, MT, TI, TJ, kModelSmagorinsky>(ctx[w.x], st, w.y, w.z, w.w, smem, ph, issued, waited, failed);
     else
-      stage_item<R, MT, TI, TJ, S64, kModelRuntime>(ctx[w.x], st, w.y, w.z, w.w, smem, ph, issued, waited, failed);
+      stage_item<R, MT, TI, TJ, kModelRuntime>(ctx[w.x], st, w.y, w.z, w.w, smem, ph, issued, waited, failed);
     if (failed) break;
   }
   if (failed) drain_after_timeout(bar, ctx[gsel].err, issued, waited, st.stall ? kStallBytes : 0u);
@@ -584,17 +565,17 @@ constexpr int TI64 = 16, TJ64 = 16;  // FP64: 320 threads, 207 KB
 // Smagorinsky build runs every grid in the build of its own model (both are
 // inlined into that kernel): a grid's state is bitwise the one it reaches
 // alone.
-template <typename R, typename MT, int TI, int TJ, bool S64 = false>
+template <typename R, typename MT, int TI, int TJ>
 cudaError_t configure_one() {
   const int bytes = (int)Cfg<R, MT, TI, TJ>::BYTES;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(k_stage<R, MT, TI, TJ, S64, kModelRuntime>, a, bytes);
+  cudaError_t e = cudaFuncSetAttribute(k_stage<R, MT, TI, TJ, kModelRuntime>, a, bytes);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_stage<R, MT, TI, TJ, S64, kModelSmagorinsky>, a, bytes);
+  e = cudaFuncSetAttribute(k_stage<R, MT, TI, TJ, kModelSmagorinsky>, a, bytes);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_stage_batch<R, MT, TI, TJ, S64, kModelSmagorinsky>, a, bytes);
+  e = cudaFuncSetAttribute(k_stage_batch<R, MT, TI, TJ, kModelSmagorinsky>, a, bytes);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_stage_batch<R, MT, TI, TJ, S64, kMixedModels>, a, bytes);
+  return cudaFuncSetAttribute(k_stage_batch<R, MT, TI, TJ, kMixedModels>, a, bytes);
 }
 
 
@@ -618,7 +599,7 @@ void fill_ctx(StageCtx<R, MT>& X, const GridDev& g) {
   X.kc = g.kc;
 }
 
-template <typename R, typename MT, int TI, int TJ, bool S64 = false>
+template <typename R, typename MT, int TI, int TJ>
 cudaError_t launch_one(const GridDev& g, int stage, int qsel, int qout, cudaStream_t s) {
   using Cf = Cfg<R, MT, TI, TJ>;
   StageCtx<R, MT> X;
@@ -627,14 +608,14 @@ cudaError_t launch_one(const GridDev& g, int stage, int qsel, int qout, cudaStre
   const int nz = g.L.hi[2] - g.L.lo[2] + 1;
   dim3 grid((g.L.hi[0] + TI) / TI, (g.L.hi[1] + TJ) / TJ, (nz + g.kc - 1) / g.kc);
   if (flow_model(X.k) == kModelSmagorinsky)
-    k_stage<R, MT, TI, TJ, S64, kModelSmagorinsky><<<grid, Cf::NT, Cf::BYTES, s>>>(X, st);
+    k_stage<R, MT, TI, TJ, kModelSmagorinsky><<<grid, Cf::NT, Cf::BYTES, s>>>(X, st);
   else
-    k_stage<R, MT, TI, TJ, S64, kModelRuntime><<<grid, Cf::NT, Cf::BYTES, s>>>(X, st);
+    k_stage<R, MT, TI, TJ, kModelRuntime><<<grid, Cf::NT, Cf::BYTES, s>>>(X, st);
   count_launches(1);
   return cudaGetLastError();
 }
 
-template <typename R, typename MT, int TI, int TJ, bool S64 = false>
+template <typename R, typename MT, int TI, int TJ>
 cudaError_t launch_batch(const void* ctx, const int4* items, int nitems, unsigned int* queue, int stage, int qsel,
                          int qout, int model, cudaStream_t s) {
   using Cf = Cfg<R, MT, TI, TJ>;
@@ -645,9 +626,9 @@ cudaError_t launch_batch(const void* ctx, const int4* items, int nitems, unsigne
   const int ctas = nitems < slots ? nitems : slots;
   const auto* X = (const StageCtx<R, MT>*)ctx;
   if (model == kModelSmagorinsky)
-    k_stage_batch<R, MT, TI, TJ, S64, kModelSmagorinsky><<<ctas, Cf::NT, Cf::BYTES, s>>>(X, items, nitems, queue, st);
+    k_stage_batch<R, MT, TI, TJ, kModelSmagorinsky><<<ctas, Cf::NT, Cf::BYTES, s>>>(X, items, nitems, queue, st);
   else
-    k_stage_batch<R, MT, TI, TJ, S64, kMixedModels><<<ctas, Cf::NT, Cf::BYTES, s>>>(X, items, nitems, queue, st);
+    k_stage_batch<R, MT, TI, TJ, kMixedModels><<<ctas, Cf::NT, Cf::BYTES, s>>>(X, items, nitems, queue, st);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -663,7 +644,7 @@ int stage_ctas_per_sm(int prec) {
 }
 
 int grid_ctas_per_sm(const GridDev& g) {
-  if (g.prec == JZ_P32 && g.variant == 2) return vr_ctas_per_sm(g.vti, g.vtj);
+  if (g.variant == 2) return vr_ctas_per_sm(g.vti, g.vtj);
   return stage_ctas_per_sm(g.prec);
 }
 
@@ -678,7 +659,6 @@ cudaError_t stage_configure() {
   if ((e = configure_one<double, double, TI64, TJ64>()) != cudaSuccess) return e;
   if ((e = configure_one<float, double, TIM, TJM>()) != cudaSuccess) return e;
   if ((e = configure_one<float, float, TI32, TJ32>()) != cudaSuccess) return e;
-  if ((e = configure_one<float, float, TI32, TJ32, true>()) != cudaSuccess) return e;
   if ((e = stage_v_configure_32x16()) != cudaSuccess) return e;
   if ((e = stage_v_configure_16x32()) != cudaSuccess) return e;
   if ((e = stage_v_configure_16x16()) != cudaSuccess) return e;
@@ -689,12 +669,12 @@ cudaError_t launch_stage(const GridDev& g, int stage, int qsel, int qout, cudaSt
   switch (g.prec) {
     case JZ_P64: return launch_one<double, double, TI64, TJ64>(g, stage, qsel, qout, s);
     case JZ_P32_M64: return launch_one<float, double, TIM, TJM>(g, stage, qsel, qout, s);
-    case JZ_P32_S64: return launch_one<float, float, TI32, TJ32, true>(g, stage, qsel, qout, s);
     default:
       if (g.variant == 2) {
         StageCtx<float, float> X;
         fill_ctx(X, g);
         const StageSel st{kRkAlpha[stage], qsel, qout, g.stall_test};
+        if (g.prec == JZ_P32_S64) return launch_stage_v_s64(X, st, s);
         if (g.vti == 16 && g.vtj == 32) return launch_stage_v_16x32(X, st, s);
         if (g.vti == 16 && g.vtj == 16) return launch_stage_v_16x16(X, st, s);
         return launch_stage_v_32x16(X, st, s);
@@ -724,8 +704,9 @@ int stage_model(const GridDev& g) { return flow_model(make_kconst<float>(g.F)); 
 cudaError_t launch_stage_batch(int prec, int variant, StageTiling tile, const void* ctx, const int4* items,
                                int nitems, unsigned int* queue, int stage, int qsel, int qout, int model,
                                cudaStream_t s) {
-  if (prec == JZ_P32 && variant == 2) {
+  if (variant == 2) {
     const StageSel st{kRkAlpha[stage], qsel, qout, 0};
+    if (prec == JZ_P32_S64) return launch_stage_v_batch_s64(ctx, items, nitems, queue, st, model, s);
     if (tile.ti == 16 && tile.tj == 32) return launch_stage_v_batch_16x32(ctx, items, nitems, queue, st, model, s);
     if (tile.ti == 16 && tile.tj == 16) return launch_stage_v_batch_16x16(ctx, items, nitems, queue, st, model, s);
     return launch_stage_v_batch_32x16(ctx, items, nitems, queue, st, model, s);
@@ -734,8 +715,6 @@ cudaError_t launch_stage_batch(int prec, int variant, StageTiling tile, const vo
     case JZ_P64: return launch_batch<double, double, TI64, TJ64>(ctx, items, nitems, queue, stage, qsel, qout, model, s);
     case JZ_P32_M64:
       return launch_batch<float, double, TIM, TJM>(ctx, items, nitems, queue, stage, qsel, qout, model, s);
-    case JZ_P32_S64:
-      return launch_batch<float, float, TI32, TJ32, true>(ctx, items, nitems, queue, stage, qsel, qout, model, s);
     default: return launch_batch<float, float, TI32, TJ32>(ctx, items, nitems, queue, stage, qsel, qout, model, s);
   }
 }

@@ -256,4 +256,8 @@ JZ_STAGE_V_DECL(32x16)
 JZ_STAGE_V_DECL(16x32)
 JZ_STAGE_V_DECL(16x16)
 #undef JZ_STAGE_V_DECL
+// the same for grids with an FP64 state between steps (16 x 16 tiles)
+cudaError_t launch_stage_v_s64(const stg::StageCtx<float, float>& X, const stg::StageSel& st, cudaStream_t s);
+cudaError_t launch_stage_v_batch_s64(const void* ctx, const int4* items, int nitems, unsigned int* queue,
+                                     const stg::StageSel& st, int model, cudaStream_t s);
 }  // namespace jz

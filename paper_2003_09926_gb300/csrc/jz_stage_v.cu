@@ -157,8 +157,10 @@ constexpr int B_RAW = 0, B_MET = 4, B_Q0 = 6, NBAR = 7;
 // own lane; the warps that share a lane quadrant take T_COLS columns each):
 // four records (primitive 5, conserved 5) of the thread's own column of
 // nodes, the state of the k march (G^k 5, low k face flux 5, lambda~, nu, J)
-// and the node's own low i and j face fluxes (10).
-constexpr int T_REC = 10, T_MARCH = 4 * T_REC, T_FACE = T_MARCH + 13, T_COLS = T_FACE + 10;
+// the node's own low i and j face fluxes (10) and, for an FP64 state between
+// steps, the node's five values of it.
+constexpr int T_REC = 10, T_MARCH = 4 * T_REC, T_FACE = T_MARCH + 13, T_Q0D = T_FACE + 10;
+constexpr int T_COLS = T_Q0D + 10;
 constexpr int T_GROUPS = (NT / 32 + 3) / 4;
 constexpr int T_ALLOC = T_GROUPS * T_COLS <= 256 ? 256 : 512;  // columns per CTA
 static_assert(T_GROUPS * T_COLS <= T_ALLOC && MINB * T_ALLOC <= 512, "tensor memory");
@@ -478,7 +480,33 @@ __device__ __forceinline__ int role_of(int tid) {
 // every wait follows from the plane index.  On a bounded-wait timeout the
 // item records where it gave up, lets its copies in flight land and returns
 // false.
-template <int MD, int ROLE>
+// Five increments in FP64, exactly.  A conversion instruction runs on the FP64
+// pipe, which passes two lanes per cycle on a GB300 SM and which the five
+// additions and roundings of an update need too; for normal numbers the
+// exponent is re-biased with integer instructions instead (one check for all
+// five: separate ones cost what they saved).  160x128x128: 0.826 and 0.750 ms
+// per step.
+__device__ __forceinline__ void widen5(const float x[5], double y[5]) {
+  bool normal = true;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) normal = normal && (__float_as_uint(x[v]) & 0x7fffffffu) - 0x00800000u < 0x7f000000u;
+  if (normal) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const uint32_t b = __float_as_uint(x[v]);
+      y[v] = __hiloint2double((int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
+    }
+  } else {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) y[v] = (double)x[v];
+  }
+}
+
+// S64: the state between time steps is FP64 (X.Q0d at the updated nodes): the
+// update adds the FP32 increment to it in FP64, stages 1-4 round their output
+// to FP32 (it feeds only the FP32 flux evaluation), and stage 5 writes both
+// the FP64 state and its FP32 copy (the next step's flux input).
+template <int MD, int ROLE, bool S64>
 __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const StageSel& st, int bx, int by, int bz,
                                        unsigned char* smem, bool first) {
   using namespace vr;
@@ -636,7 +664,7 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
   // Q^(0) of the plane being updated: for the first stage it is the stage
   // input, which the own column's records hold; otherwise TMA stages it one
   // plane ahead (tile rows, 36 columns from the aligned column i0-2)
-  const bool q0_own = st.qin == 0;
+  const bool q0_own = S64 || st.qin == 0;
   const float* q0buf = reinterpret_cast<const float*>(smem + O_Q0);
   auto issue_q0 = [&](int p) {
     if (ROLE == 0 && tid == 0 && !q0_own) {
@@ -748,6 +776,8 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
         tie(qd);
         tie(qp);
         tm_ld10(tm + T_FACE, hl);
+        float q0w[10];  // the FP64 values' words
+        if constexpr (S64) tm_ld10(tm + T_Q0D, q0w);
         face_v(c, make_float2(mv[10], mv[11]), make_float2(lt3n, nu3n), mv, G3n, qc, qd, qb, qp, hk);
         {
           float nv[13];
@@ -768,9 +798,13 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
         ld5j(sm.Hj4, sm.Hj1, ny + 1, nx, hj);
         tm_wait_ld();
         tie(hl);
+        if constexpr (S64) tie(q0w);
         if (own && t >= t0) {
           float q0[5];
-          if (q0_own) {
+          if constexpr (S64) {  // the increment alone
+#pragma unroll
+            for (int v = 0; v < 5; ++v) q0[v] = 0.f;
+          } else if (q0_own) {
 #pragma unroll
             for (int v = 0; v < 5; ++v) q0[v] = qd[v];
           } else {
@@ -791,8 +825,22 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
             qn[v + 1] = r.y;
           }
           qn[4] = fmaf(aj, ((hi[4] - hl[4]) + (hj[4] - hl[9])) + (hk[4] - mv[9]), q0[4]);
+          if constexpr (S64) {
+            double* const dst64 = X.Q0d + n_t0 + (long long)(t - t0) * L.plane;
+            double qd[5];
+            widen5(qn, qd);
 #pragma unroll
-          for (int v = 0; v < 5; ++v) dst[v * npad] = qn[v];
+            for (int v = 0; v < 5; ++v)
+              qd[v] += __hiloint2double(__float_as_int(q0w[2 * v + 1]), __float_as_int(q0w[2 * v]));
+#pragma unroll
+            for (int v = 0; v < 5; ++v) {
+              dst[v * npad] = (float)qd[v];
+              if (st.qout == 0) dst64[v * npad] = qd[v];
+            }
+          } else {
+#pragma unroll
+            for (int v = 0; v < 5; ++v) dst[v * npad] = qn[v];
+          }
         }
       }
       __syncwarp();
@@ -805,6 +853,14 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
       // A tile node keeps its two faces in tensor memory for its residual.
       if (live) {
         issue_q0(t + 1);
+        // the FP64 state of plane t+1, through tensor memory to its update: the
+        // faces hide the loads' latency
+        double q0d[S64 ? 5 : 1];
+        if constexpr (S64 && ROLE == 0) {
+          const double* src = X.Q0d + n_t0 + (long long)(t + 1 - t0) * L.plane;
+#pragma unroll
+          for (int v = 0; v < 5; ++v) q0d[v] = own ? src[v * npad] : 0.0;
+        }
         const float4* qv = sm.QV + r1;
         const float* qe = sm.QE + r1;
         float qo[5], hij[10];
@@ -832,6 +888,15 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
         }
         if constexpr (ROLE == 0) {
           tm_st10(tm + T_FACE, hij);
+          if constexpr (S64) {
+            float q0w[10];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) {
+              q0w[2 * v] = __int_as_float(__double2loint(q0d[v]));
+              q0w[2 * v + 1] = __int_as_float(__double2hiint(q0d[v]));
+            }
+            tm_st10(tm + T_Q0D, q0w);
+          }
         }
       }
       if (t + 3 <= t1 + 1) {
@@ -865,20 +930,20 @@ fail:
   return false;
 }
 
-template <int MD>
+template <int MD, bool S64>
 __global__ void __launch_bounds__(vr::NT, vr::MINB)
     k_stage_v(const __grid_constant__ StageCtx<float, float> X, const StageSel st) {
   extern __shared__ __align__(128) unsigned char smem[];
   tm_alloc(smem);
   switch (role_of(threadIdx.x)) {
-    case 0: item_v<MD, 0>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
-    case 2: item_v<MD, 2>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
-    default: item_v<MD, 1>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
+    case 0: item_v<MD, 0, S64>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
+    case 2: item_v<MD, 2, S64>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
+    default: item_v<MD, 1, S64>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
   }
   tm_free(smem);
 }
 
-template <int MD>
+template <int MD, bool S64>
 __global__ void __launch_bounds__(vr::NT, vr::MINB)
     k_stage_v_batch(const StageCtx<float, float>* __restrict__ ctx, const int4* __restrict__ items, int nitems,
                     unsigned int* queue, const StageSel st) {
@@ -895,9 +960,9 @@ __global__ void __launch_bounds__(vr::NT, vr::MINB)
     const int4 w = items[it];
     bool ok;
     switch (role_of(threadIdx.x)) {
-      case 0: ok = item_v<MD, 0>(ctx[w.x], st, w.y, w.z, w.w, smem, first); break;
-      case 2: ok = item_v<MD, 2>(ctx[w.x], st, w.y, w.z, w.w, smem, first); break;
-      default: ok = item_v<MD, 1>(ctx[w.x], st, w.y, w.z, w.w, smem, first); break;
+      case 0: ok = item_v<MD, 0, S64>(ctx[w.x], st, w.y, w.z, w.w, smem, first); break;
+      case 2: ok = item_v<MD, 2, S64>(ctx[w.x], st, w.y, w.z, w.w, smem, first); break;
+      default: ok = item_v<MD, 1, S64>(ctx[w.x], st, w.y, w.z, w.w, smem, first); break;
     }
     if (!ok) break;
     first = false;
@@ -905,56 +970,84 @@ __global__ void __launch_bounds__(vr::NT, vr::MINB)
   tm_free(smem);
 }
 
-template <int MD>
+template <int MD, bool S64>
 cudaError_t configure_model() {
-  cudaError_t e = cudaFuncSetAttribute(k_stage_v<MD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vr::BYTES);
+  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(k_stage_v<MD, S64>, at, (int)vr::BYTES);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_stage_v_batch<MD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vr::BYTES);
+  return cudaFuncSetAttribute(k_stage_v_batch<MD, S64>, at, (int)vr::BYTES);
+}
+
+template <int MD, bool S64>
+cudaError_t launch(const StageCtx<float, float>& X, const StageSel& st, cudaStream_t s) {
+  const Layout& L = X.L;
+  const int nz = L.hi[2] - L.lo[2] + 1;
+  dim3 grid((L.hi[0] + vr::TI) / vr::TI, (L.hi[1] + vr::TJ) / vr::TJ, (nz + X.kc - 1) / X.kc);
+  k_stage_v<MD, S64><<<grid, vr::NT, vr::BYTES, s>>>(X, st);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+template <int MD, bool S64>
+cudaError_t launch_batch(const void* ctx, const int4* items, int nitems, unsigned int* queue, const StageSel& st,
+                         cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(unsigned int), s);
+  if (e != cudaSuccess) return e;
+  const int slots = device_sm_count() * vr::MINB;
+  const int ctas = nitems < slots ? nitems : slots;
+  k_stage_v_batch<MD, S64><<<ctas, vr::NT, vr::BYTES, s>>>((const StageCtx<float, float>*)ctx, items, nitems, queue, st);
+  count_launches(1);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t VR_FN(stage_v_configure)() {
   cudaError_t e;
-  if ((e = configure_model<kModelRuntime>()) != cudaSuccess) return e;
-  if ((e = configure_model<kModelSmagorinsky>()) != cudaSuccess) return e;
-  if ((e = configure_model<kModelVreman>()) != cudaSuccess) return e;
-  return configure_model<kModelEuler>();
+#if VR_TI == 16 && VR_TJ == 16
+  if ((e = configure_model<kModelRuntime, true>()) != cudaSuccess) return e;
+  if ((e = configure_model<kModelSmagorinsky, true>()) != cudaSuccess) return e;
+#endif
+  if ((e = configure_model<kModelRuntime, false>()) != cudaSuccess) return e;
+  if ((e = configure_model<kModelSmagorinsky, false>()) != cudaSuccess) return e;
+  if ((e = configure_model<kModelVreman, false>()) != cudaSuccess) return e;
+  return configure_model<kModelEuler, false>();
 }
 
 cudaError_t VR_FN(launch_stage_v)(const StageCtx<float, float>& X, const StageSel& st, cudaStream_t s) {
-  const Layout& L = X.L;
-  const int nz = L.hi[2] - L.lo[2] + 1;
-  dim3 grid((L.hi[0] + vr::TI) / vr::TI, (L.hi[1] + vr::TJ) / vr::TJ, (nz + X.kc - 1) / X.kc);
   switch (flow_model(X.k)) {
-    case kModelSmagorinsky: k_stage_v<kModelSmagorinsky><<<grid, vr::NT, vr::BYTES, s>>>(X, st); break;
-    case kModelVreman: k_stage_v<kModelVreman><<<grid, vr::NT, vr::BYTES, s>>>(X, st); break;
-    case kModelEuler: k_stage_v<kModelEuler><<<grid, vr::NT, vr::BYTES, s>>>(X, st); break;
-    default: k_stage_v<kModelRuntime><<<grid, vr::NT, vr::BYTES, s>>>(X, st); break;
+    case kModelSmagorinsky: return launch<kModelSmagorinsky, false>(X, st, s);
+    case kModelVreman: return launch<kModelVreman, false>(X, st, s);
+    case kModelEuler: return launch<kModelEuler, false>(X, st, s);
+    default: return launch<kModelRuntime, false>(X, st, s);
   }
-  count_launches(1);
-  return cudaGetLastError();
 }
 
 // model: the flow model every grid of the batch shares (kModelRuntime when
 // they differ)
 cudaError_t VR_FN(launch_stage_v_batch)(const void* ctx, const int4* items, int nitems, unsigned int* queue,
                                         const StageSel& st, int model, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(unsigned int), s);
-  if (e != cudaSuccess) return e;
-  const int slots = device_sm_count() * vr::MINB;
-  const int ctas = nitems < slots ? nitems : slots;
-  const auto* X = (const StageCtx<float, float>*)ctx;
   switch (model) {
-    case kModelSmagorinsky:
-      k_stage_v_batch<kModelSmagorinsky><<<ctas, vr::NT, vr::BYTES, s>>>(X, items, nitems, queue, st);
-      break;
-    case kModelVreman: k_stage_v_batch<kModelVreman><<<ctas, vr::NT, vr::BYTES, s>>>(X, items, nitems, queue, st); break;
-    case kModelEuler: k_stage_v_batch<kModelEuler><<<ctas, vr::NT, vr::BYTES, s>>>(X, items, nitems, queue, st); break;
-    default: k_stage_v_batch<kModelRuntime><<<ctas, vr::NT, vr::BYTES, s>>>(X, items, nitems, queue, st); break;
+    case kModelSmagorinsky: return launch_batch<kModelSmagorinsky, false>(ctx, items, nitems, queue, st, s);
+    case kModelVreman: return launch_batch<kModelVreman, false>(ctx, items, nitems, queue, st, s);
+    case kModelEuler: return launch_batch<kModelEuler, false>(ctx, items, nitems, queue, st, s);
+    default: return launch_batch<kModelRuntime, false>(ctx, items, nitems, queue, st, s);
   }
-  count_launches(1);
-  return cudaGetLastError();
 }
+
+#if VR_TI == 16 && VR_TJ == 16
+// JZ_P32_S64 grids: one tile shape, and constant flags for the Smagorinsky
+// model of the configurations only
+cudaError_t launch_stage_v_s64(const StageCtx<float, float>& X, const StageSel& st, cudaStream_t s) {
+  if (flow_model(X.k) == kModelSmagorinsky) return launch<kModelSmagorinsky, true>(X, st, s);
+  return launch<kModelRuntime, true>(X, st, s);
+}
+
+cudaError_t launch_stage_v_batch_s64(const void* ctx, const int4* items, int nitems, unsigned int* queue,
+                                     const StageSel& st, int model, cudaStream_t s) {
+  if (model == kModelSmagorinsky) return launch_batch<kModelSmagorinsky, true>(ctx, items, nitems, queue, st, s);
+  return launch_batch<kModelRuntime, true>(ctx, items, nitems, queue, st, s);
+}
+#endif
 
 }  // namespace jz
