@@ -20,7 +20,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # (source, object, extra defines): the FP32 vector-record stage kernel is
 # built once per tile shape the autotuner may choose
 SOURCES = [(s, s.replace(".cu", ".o"), []) for s in
-           ("jz_api.cu", "jz_grid.cu", "jz_reduce.cu", "jz_stage.cu", "jz_static.cu", "jz_peak.cu", "jz_stats.cu")]
+           ("jz_api.cu", "jz_grid.cu", "jz_reduce.cu", "jz_stage.cu", "jz_stage_d.cu", "jz_static.cu", "jz_peak.cu", "jz_stats.cu")]
 SOURCES += [("jz_stage_v.cu", f"jz_stage_v_{ti}x{tj}.o", [f"-DVR_TI={ti}", f"-DVR_TJ={tj}"])
             for ti, tj in ((32, 16), (16, 32), (16, 16))]
 

@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(Cfg<R, MT, TI, TJ>::NT, Cfg<R, MT, TI, TJ>::MI
 // share outweighs the overlap of the two CTAs' barriers)
 constexpr int TI32 = 32, TJ32 = 16;  // P32: 608 threads, 191 KB: one CTA per SM
 constexpr int TIM = 32, TJM = 16;    // P32_M64: 608 threads, 220 KB (FP64 metric staging): one CTA per SM
-constexpr int TI64 = 16, TJ64 = 16;  // FP64: 320 threads, 207 KB
+constexpr int TI64 = 16, TJ64 = 16;  // FP64 (jz_stage_d.cu)
 
 // The scalar kernels are built for two flow models: the configurations'
 // (Smagorinsky, sigma = 1/2) with constant flags, and every other with the
@@ -637,7 +637,7 @@ cudaError_t launch_batch(const void* ctx, const int4* items, int nitems, unsigne
 
 int stage_ctas_per_sm(int prec) {
   switch (prec) {
-    case JZ_P64: return Cfg<double, double, TI64, TJ64>::MINB;
+    case JZ_P64: return stage_d_ctas_per_sm({TI64, TJ64});
     case JZ_P32_M64: return Cfg<float, double, TIM, TJM>::MINB;
     default: return Cfg<float, float, TI32, TJ32>::MINB;
   }
@@ -656,7 +656,7 @@ StageTiling stage_tiling(int prec) {
 
 cudaError_t stage_configure() {
   cudaError_t e;
-  if ((e = configure_one<double, double, TI64, TJ64>()) != cudaSuccess) return e;
+  if ((e = stage_d_configure()) != cudaSuccess) return e;
   if ((e = configure_one<float, double, TIM, TJM>()) != cudaSuccess) return e;
   if ((e = configure_one<float, float, TI32, TJ32>()) != cudaSuccess) return e;
   if ((e = stage_v_configure_32x16()) != cudaSuccess) return e;
@@ -667,7 +667,11 @@ cudaError_t stage_configure() {
 
 cudaError_t launch_stage(const GridDev& g, int stage, int qsel, int qout, cudaStream_t s) {
   switch (g.prec) {
-    case JZ_P64: return launch_one<double, double, TI64, TJ64>(g, stage, qsel, qout, s);
+    case JZ_P64: {
+      StageCtx<double, double> X;
+      fill_ctx(X, g);
+      return launch_stage_d(X, StageSel{kRkAlpha[stage], qsel, qout, g.stall_test}, grid_tiling(g), s);
+    }
     case JZ_P32_M64: return launch_one<float, double, TIM, TJM>(g, stage, qsel, qout, s);
     default:
       if (g.variant == 2) {
@@ -712,7 +716,8 @@ cudaError_t launch_stage_batch(int prec, int variant, StageTiling tile, const vo
     return launch_stage_v_batch_32x16(ctx, items, nitems, queue, st, model, s);
   }
   switch (prec) {
-    case JZ_P64: return launch_batch<double, double, TI64, TJ64>(ctx, items, nitems, queue, stage, qsel, qout, model, s);
+    case JZ_P64:
+      return launch_stage_d_batch(ctx, items, nitems, queue, StageSel{kRkAlpha[stage], qsel, qout, 0}, tile, model, s);
     case JZ_P32_M64:
       return launch_batch<float, double, TIM, TJM>(ctx, items, nitems, queue, stage, qsel, qout, model, s);
     default: return launch_batch<float, float, TI32, TJ32>(ctx, items, nitems, queue, stage, qsel, qout, model, s);

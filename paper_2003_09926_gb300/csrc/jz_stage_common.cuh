@@ -256,7 +256,14 @@ JZ_STAGE_V_DECL(32x16)
 JZ_STAGE_V_DECL(16x32)
 JZ_STAGE_V_DECL(16x16)
 #undef JZ_STAGE_V_DECL
-// the same for grids with an FP64 state between steps (16 x 16 tiles)
+// FP64 kernel (jz_stage_d.cu)
+cudaError_t stage_d_configure();
+int stage_d_ctas_per_sm(StageTiling t);
+cudaError_t launch_stage_d(const stg::StageCtx<double, double>& X, const stg::StageSel& st, StageTiling t,
+                           cudaStream_t s);
+cudaError_t launch_stage_d_batch(const void* ctx, const int4* items, int nitems, unsigned int* queue,
+                                 const stg::StageSel& st, StageTiling t, int model, cudaStream_t s);
+// the FP32 record kernel for grids with an FP64 state between steps (16 x 16 tiles)
 cudaError_t launch_stage_v_s64(const stg::StageCtx<float, float>& X, const stg::StageSel& st, cudaStream_t s);
 cudaError_t launch_stage_v_batch_s64(const void* ctx, const int4* items, int nitems, unsigned int* queue,
                                      const stg::StageSel& st, int model, cudaStream_t s);
