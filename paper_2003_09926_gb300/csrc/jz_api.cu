@@ -452,7 +452,14 @@ int create_grid(const jz_grid_desc* desc, const int* o0, const int* o1, void* de
   d.variant = (d.prec == JZ_P32 || d.prec == JZ_P32_S64) ? 2 : 0;  // the vector-record kernel where it is built
   d.vti = 16;  // two CTAs per SM; as fast as 32 x 16 on 256x192x192, faster on small grids
   d.vtj = 16;
-  d.kc = default_kc(cv.L, grid_tiling(d), grid_ctas_per_sm(d));
+  if (d.prec == JZ_P64) {
+    StageTiling t{16, 16};
+    stage_d_split(cv.L, t, d.kc);
+    d.vti = t.ti;
+    d.vtj = t.tj;
+  } else {
+    d.kc = default_kc(cv.L, grid_tiling(d), grid_ctas_per_sm(d));
+  }
   d.kc_set = 0;
   const int gn[3] = {desc->ni, desc->nj, desc->nk};
   for (int a = 0; a < 3; ++a) {
@@ -887,6 +894,10 @@ struct BatchPlan {
   int xbegin[3] = {0, 0, 0}, xcount[3] = {0, 0, 0}, xblocks = 1;
 };
 
+// the tile of a batch's work items: every grid's, and 16 x 16 for FP64 grids,
+// which alone may run 8 x 8 tiles to fill the chip
+StageTiling batch_tiling(const GridDev& d) { return d.prec == JZ_P64 ? StageTiling{16, 16} : grid_tiling(d); }
+
 // k-chunk lengths of the grids of a batch.  A grid stepped alone is cut into
 // chunks short enough to fill the device by itself; in a batch the other
 // grids do that, and every chunk costs about three planes more than it
@@ -912,7 +923,10 @@ void batch_chunks(jz_grid* const* grids, int n, StageTiling t, std::vector<int>&
     longest = std::max(longest, g[k].nz);
   }
   std::stable_sort(g.begin(), g.end(), [](const G& a, const G& b) { return a.work > b.work; });
-  const long long slots = (long long)device_sm_count() * grid_ctas_per_sm(grids[0]->dev);
+  GridDev d0 = grids[0]->dev;
+  d0.vti = t.ti;
+  d0.vtj = t.tj;
+  const long long slots = (long long)device_sm_count() * grid_ctas_per_sm(d0);
   auto chunk = [](const G& x, int len) {
     if (x.fixed) return x.fixed;
     const int c = (x.nz + len - 1) / len;
@@ -961,9 +975,9 @@ int batch_plan(jz_grid* const* grids, int n, BatchPlan& P) {
     if (prec >= 0 && grids[k]->dev.prec != prec) return fail(JZ_EINVAL, "batch grids must share one precision mode");
     prec = grids[k]->dev.prec;
   }
-  const StageTiling t = grid_tiling(grids[0]->dev);
+  const StageTiling t = batch_tiling(grids[0]->dev);
   for (int k = 1; k < n; ++k) {
-    const StageTiling u = grid_tiling(grids[k]->dev);
+    const StageTiling u = batch_tiling(grids[k]->dev);
     if (grids[k]->dev.variant != grids[0]->dev.variant || u.ti != t.ti || u.tj != t.tj)
       return fail(JZ_EINVAL, "batch grids must share one stage kernel and tile shape");
   }
@@ -1087,7 +1101,7 @@ int enqueue_batch_step(jz_batch* b, double cfl) {
   if (e != cudaSuccess) return fail(JZ_ECUDA, "batched time step launch failed: %s", cudaGetErrorString(e));
   const int src[5] = {0, 1, 2, 1, 2}, out[5] = {1, 2, 1, 2, 0};
   for (int l = 0; l < 5; ++l) {
-    e = launch_stage_batch(b->prec, b->grids[0]->dev.variant, grid_tiling(b->grids[0]->dev), b->dev + b->off_stage,
+    e = launch_stage_batch(b->prec, b->grids[0]->dev.variant, batch_tiling(b->grids[0]->dev), b->dev + b->off_stage,
                            (const int4*)(b->dev + b->off_items), b->nitems, (unsigned int*)(b->dev + b->off_queue), l,
                            src[l], out[l], b->model, s);
     if (e != cudaSuccess) return fail(JZ_ECUDA, "batched stage launch failed: %s", cudaGetErrorString(e));
@@ -1114,6 +1128,12 @@ int create_batch(jz_grid* const* grids, int n, bool coupled, void* dev_buf, size
   for (int k = 0; k < n; ++k) {
     GridDev d = grids[k]->dev;
     d.kc = P.kc[k];
+    const StageTiling t = batch_tiling(d), own = grid_tiling(d);
+    if (own.ti != t.ti || own.tj != t.tj) {  // TMA maps for the batch's tile
+      d.vti = t.ti;
+      d.vtj = t.tj;
+      if (int rc = build_maps(d)) return rc;
+    }
     stage_ctx_fill(host.data() + P.off_stage + (size_t)k * stage_ctx_bytes(prec), d);
     bc_ctx_fill(host.data() + P.off_bc + (size_t)k * bc_ctx_bytes(), grids[k]->dev);
     rate_ctx_fill(host.data() + P.off_rate + (size_t)k * rate_ctx_bytes(), grids[k]->dev);

@@ -30,7 +30,7 @@ struct GridDev {
   int kc_set;          // kc was set by the caller (a batch then keeps it)
   int goff[3], gn[3];  // global index of local node 0 and global node counts (blocks; else 0 and n)
   int variant;         // stage kernel: 2 vector records (P32 by default, P32_S64), 0 scalar records
-  int vti, vtj;        // tile shape of the vector-record kernel (32 x 16, 16 x 32 or 16 x 16)
+  int vti, vtj;        // tile shape of the vector-record kernel (32 x 16, 16 x 32 or 16 x 16) or of the FP64 kernel (16 x 16, 8 x 8)
   int stall_test;      // test only: the stage kernels' copies wait for bytes that nothing delivers
   int step_diag;       // each step's time-step reduction also forms the diagnostics of the state it reads
   CUtensorMap tmQ[3];  // TMA maps of Q0, QA, QB (stage kernel tile box)
@@ -117,10 +117,12 @@ cudaError_t launch_timestep_batch(int prec, const void* ctx, int n, double cfl, 
 struct StageTiling { int ti, tj; };
 StageTiling stage_tiling(int prec);
 // the tile of the kernel a grid runs: its chosen shape for the FP32
-// vector-record kernel, else the fixed tile of its precision mode
+// vector-record and the FP64 kernel, else the fixed tile of its precision mode
 inline StageTiling grid_tiling(const GridDev& g) {
-  return g.variant == 2 ? StageTiling{g.vti, g.vtj} : stage_tiling(g.prec);
+  return g.variant == 2 || g.prec == JZ_P64 ? StageTiling{g.vti, g.vtj} : stage_tiling(g.prec);
 }
+// the FP64 kernel's tile and k-chunk length for a grid
+void stage_d_split(const Layout& L, StageTiling& t, int& kc);
 int stage_ctas_per_sm(int prec);
 // resident CTAs per SM of the stage kernel a grid runs
 int grid_ctas_per_sm(const GridDev& g);

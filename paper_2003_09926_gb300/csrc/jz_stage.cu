@@ -556,7 +556,6 @@ __global__ void __launch_bounds__(Cfg<R, MT, TI, TJ>::NT, Cfg<R, MT, TI, TJ>::MI
 // share outweighs the overlap of the two CTAs' barriers)
 constexpr int TI32 = 32, TJ32 = 16;  // P32: 608 threads, 191 KB: one CTA per SM
 constexpr int TIM = 32, TJM = 16;    // P32_M64: 608 threads, 220 KB (FP64 metric staging): one CTA per SM
-constexpr int TI64 = 16, TJ64 = 16;  // FP64 (jz_stage_d.cu)
 
 // The scalar kernels are built for two flow models: the configurations'
 // (Smagorinsky, sigma = 1/2) with constant flags, and every other with the
@@ -637,19 +636,18 @@ cudaError_t launch_batch(const void* ctx, const int4* items, int nitems, unsigne
 
 int stage_ctas_per_sm(int prec) {
   switch (prec) {
-    case JZ_P64: return stage_d_ctas_per_sm({TI64, TJ64});
     case JZ_P32_M64: return Cfg<float, double, TIM, TJM>::MINB;
     default: return Cfg<float, float, TI32, TJ32>::MINB;
   }
 }
 
 int grid_ctas_per_sm(const GridDev& g) {
+  if (g.prec == JZ_P64) return stage_d_ctas_per_sm({g.vti, g.vtj});
   if (g.variant == 2) return vr_ctas_per_sm(g.vti, g.vtj);
   return stage_ctas_per_sm(g.prec);
 }
 
 StageTiling stage_tiling(int prec) {
-  if (prec == JZ_P64) return {TI64, TJ64};
   if (prec == JZ_P32_M64) return {TIM, TJM};
   return {TI32, TJ32};
 }
@@ -717,7 +715,7 @@ cudaError_t launch_stage_batch(int prec, int variant, StageTiling tile, const vo
   }
   switch (prec) {
     case JZ_P64:
-      return launch_stage_d_batch(ctx, items, nitems, queue, StageSel{kRkAlpha[stage], qsel, qout, 0}, tile, model, s);
+      return launch_stage_d_batch(ctx, items, nitems, queue, StageSel{kRkAlpha[stage], qsel, qout, 0}, model, s);
     case JZ_P32_M64:
       return launch_batch<float, double, TIM, TJM>(ctx, items, nitems, queue, stage, qsel, qout, model, s);
     default: return launch_batch<float, float, TI32, TJ32>(ctx, items, nitems, queue, stage, qsel, qout, model, s);

@@ -262,7 +262,7 @@ int stage_d_ctas_per_sm(StageTiling t);
 cudaError_t launch_stage_d(const stg::StageCtx<double, double>& X, const stg::StageSel& st, StageTiling t,
                            cudaStream_t s);
 cudaError_t launch_stage_d_batch(const void* ctx, const int4* items, int nitems, unsigned int* queue,
-                                 const stg::StageSel& st, StageTiling t, int model, cudaStream_t s);
+                                 const stg::StageSel& st, int model, cudaStream_t s);
 // the FP32 record kernel for grids with an FP64 state between steps (16 x 16 tiles)
 cudaError_t launch_stage_v_s64(const stg::StageCtx<float, float>& X, const stg::StageSel& st, cudaStream_t s);
 cudaError_t launch_stage_v_batch_s64(const void* ctx, const int4* items, int nitems, unsigned int* queue,

@@ -119,11 +119,11 @@ struct Cfg {
   static constexpr size_t O_GJ = O_GI + al(8 * 7 * TJ * GIW);
   static constexpr size_t O_HI = O_GJ + al(8 * 7 * GJH * TI);  // face fluxes
   static constexpr size_t O_HJ = O_HI + al(8 * 5 * TJ * HIW);
-  static constexpr size_t O_BAR = O_HJ + al(8 * 5 * HJH * TI);
+  static constexpr size_t O_SCR = O_GI;  // a chunk's first three planes are staged over the node and face buffers
+  static constexpr size_t O_END = O_HJ + al(8 * 5 * HJH * TI);
+  static constexpr size_t O_BAR = O_END > O_SCR + 3 * RAW_B ? O_END : O_SCR + 3 * RAW_B;
   static constexpr size_t O_TMEM = O_BAR + 64;
   static constexpr size_t BYTES = O_BAR + 128;
-  static constexpr size_t O_SCR = O_GI;  // a chunk's first three planes are staged over the node and face buffers
-  static_assert(O_BAR - O_SCR >= 3 * RAW_B, "prologue staging does not fit");
   static_assert(BYTES <= 232448, "shared memory");
   static constexpr uint32_t RAW_TX = 8 * 5 * PL, MET_TX = 8 * 10 * MPL, Q0_TX = 8 * 5 * UPL;
   // tensor memory, 32-bit columns per warp group: four records of the own
@@ -705,7 +705,11 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
   tm_free<C>(smem);
 }
 
+// Tiles: 16 x 16 (one CTA per SM) costs 15.2 FP64 warp instructions per node
+// and plane, halo included; 8 x 8 (three CTAs) 17.3, but cuts a small grid
+// into enough CTAs for the whole chip.
 using Big = Cfg<16, 16>;
+using Small = Cfg<8, 8>;
 
 template <class C, int MD>
 cudaError_t configure() {
@@ -741,19 +745,54 @@ cudaError_t launch_batch(const void* ctx, const int4* items, int nitems, unsigne
 
 cudaError_t stage_d_configure() {
   cudaError_t e;
+  if ((e = configure<Small, kModelSmagorinsky>()) != cudaSuccess) return e;
+  if ((e = configure<Small, kModelRuntime>()) != cudaSuccess) return e;
   if ((e = configure<Big, kModelSmagorinsky>()) != cudaSuccess) return e;
   return configure<Big, kModelRuntime>();
 }
 
-int stage_d_ctas_per_sm(StageTiling) { return Big::MINB; }
+int stage_d_ctas_per_sm(StageTiling t) { return t.ti == Small::TI ? Small::MINB : Big::MINB; }
 
-cudaError_t launch_stage_d(const StageCtx<double, double>& X, const StageSel& st, StageTiling, cudaStream_t s) {
+// The tile and k-chunk length of a grid: the split with the least modelled time
+// (microseconds, fitted to measured stages).
+//   16 x 16: the CTAs of an SM run one after the other, a chunk of kc planes
+//     takes 33.8 kc + 45 (45: its prologue and the two planes that build up the
+//     march), the FP64 pipe 92% busy.
+//   8 x 8: only while all CTAs are resident together; a plane takes
+//     9.5 + 7 c for c CTAs per SM and 15.6 at least (one CTA's three warps
+//     wait for one another's results half of the time).
+// 48x32x32: 8 x 8 with chunks of 3 planes 93 us per stage (2: 99, 5: 108),
+// 16 x 16 with chunks of 2 115 us.  77x42x54: 262 and 250 us.
+void stage_d_split(const Layout& L, StageTiling& t, int& kc) {
+  const int nz = L.hi[2] - L.lo[2] + 1;
+  const long long sms = device_sm_count();
+  auto tiles = [&](int n) { return (long long)((L.hi[0] + n) / n) * ((L.hi[1] + n) / n); };
+  const long long big = tiles(Big::TI), small = tiles(Small::TI);
+  double best = 1e300;
+  auto take = [&](double cost, int n, int k) {
+    if (cost >= best * (1.0 - 1e-9)) return;
+    best = cost;
+    t = {n, n};
+    kc = k;
+  };
+  for (int k = 1; k <= nz; ++k) {
+    const int chunks = (nz + k - 1) / k;
+    take((double)((big * chunks + sms - 1) / sms) * (33.8 * k + 45.0), Big::TI, k);
+    const double c = (double)(small * chunks) / (double)sms;
+    if (small * chunks <= sms * Small::MINB) take(std::fmax(15.6, 9.5 + 7.0 * c) * (k + 1.7) + 8.0, Small::TI, k);
+  }
+}
+
+cudaError_t launch_stage_d(const StageCtx<double, double>& X, const StageSel& st, StageTiling t, cudaStream_t s) {
+  if (t.ti == Small::TI)
+    return flow_model(X.k) == kModelSmagorinsky ? launch<Small, kModelSmagorinsky>(X, st, s)
+                                                : launch<Small, kModelRuntime>(X, st, s);
   return flow_model(X.k) == kModelSmagorinsky ? launch<Big, kModelSmagorinsky>(X, st, s)
                                               : launch<Big, kModelRuntime>(X, st, s);
 }
 
 cudaError_t launch_stage_d_batch(const void* ctx, const int4* items, int nitems, unsigned int* queue,
-                                 const StageSel& st, StageTiling, int model, cudaStream_t s) {
+                                 const StageSel& st, int model, cudaStream_t s) {
   return model == kModelSmagorinsky ? launch_batch<Big, kModelSmagorinsky>(ctx, items, nitems, queue, st, s)
                                     : launch_batch<Big, kModelRuntime>(ctx, items, nitems, queue, st, s);
 }
