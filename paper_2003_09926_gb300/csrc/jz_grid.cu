@@ -282,140 +282,125 @@ Slabs make_slabs(const int ol[3], const int oh[3], const int il[3], const int ih
   return s;
 }
 
-__device__ __forceinline__ bool slab_node(const Slabs& sl, int q, int t, int& i, int& j, int& k) {
-  const int e0 = sl.e[q][0], e1 = sl.e[q][1];
-  if (t >= e0 * e1 * sl.e[q][2]) return false;
-  i = sl.a[q][0] + t % e0;
-  j = sl.a[q][1] + (t / e0) % e1;
-  k = sl.a[q][2] + t / (e0 * e1);
+// The value of the padded node (i, j, k) outside the updated box: that of the
+// grid node its index maps to (wrap, clamp for the ghost layers behind a face,
+// or across the centreline of a cylindrical grid): a copy when that node is
+// updated by the stages, its boundary-condition value (computed here from the
+// interior node it reads, or, on the centreline, from the azimuthal means)
+// when it is a boundary node.  Only updated nodes are read.  False for a node
+// that is left alone: a ghost behind an exchange face (the halo exchange's)
+// and, with AXIS_IN, a centreline node (its mean's own block writes it).
+template <typename ST, typename MT, bool FAST, bool AXIS_IN>
+__device__ __forceinline__ bool node_value(const Layout& L, const double* inflow, const double* axis, const FlowC& F,
+                                           const ST* Q, const MT* __restrict__ M, int i, int j, int k, ST v[5]) {
+  if ((i < 0 && L.bc[0] == BC_EXCHANGE) || (i >= L.n[0] && L.bc[1] == BC_EXCHANGE) ||
+      (j < 0 && L.bc[2] == BC_EXCHANGE) || (j >= L.n[1] && L.bc[3] == BC_EXCHANGE) ||
+      (k < 0 && L.bc[4] == BC_EXCHANGE) || (k >= L.n[2] && L.bc[5] == BC_EXCHANGE))
+    return false;
+  int mi = i, mj = j, mk = k;
+  L.map_node(mi, mj, mk);
+  if (mi >= L.lo[0] && mi <= L.hi[0] && mj >= L.lo[1] && mj <= L.hi[1] && mk >= L.lo[2] && mk <= L.hi[2]) {
+    const long long src = L.at(mi, mj, mk);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) v[c] = Q[(long long)c * L.npad + src];
+    return true;
+  }
+  // boundary node (mi, mj, mk): the face latest in the order y-, y+, z-, z+,
+  // x+, x- decides
+  const int idx[3] = {mi, mj, mk};
+  const int order[6] = {2, 3, 4, 5, 1, 0};
+  int f = -1;
+#pragma unroll
+  for (int o = 0; o < 6; ++o) {
+    const int ff = order[o], d = ff / 2;
+    if (L.bc[ff] == BC_PERIODIC || L.bc[ff] == BC_EXCHANGE) continue;
+    if (idx[d] == ((ff % 2 == 0) ? 0 : L.n[d] - 1)) f = ff;
+  }
+  if (f < 0) return false;  // not reached: a node outside the updated box lies on some face
+  if (L.bc[f] == BC_INFLOW) {  // x- face only: profile tabulated per (j, k)
+    to_conserved<ST, FAST>(flow_const<ST>(F.gm1, F.gm1_f), ST(1), (ST)inflow[mk * L.n[1] + mj], ST(0), ST(0),
+                           flow_const<ST>(1.0 / F.gamma, F.pe_f), v);
+    return true;
+  }
+  if (L.bc[f] == BC_AXIS) {  // azimuthal mean of the adjacent radial line
+    if (AXIS_IN) return false;
+#pragma unroll
+    for (int c = 0; c < 5; ++c) v[c] = (ST)axis[c * L.n[0] + mi];
+    return true;
+  }
+  // far field: nearest updated node, normal at the boundary node (on the
+  // centreline the face metric vanishes: that of the adjacent radial node)
+  int ci[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) ci[d] = idx[d] < L.lo[d] ? L.lo[d] : (idx[d] > L.hi[d] ? L.hi[d] : idx[d]);
+  const long long src = L.at(ci[0], ci[1], ci[2]);
+  const long long nb = L.at(mi, (L.cyl && mj == 0) ? 1 : mj, mk);
+  const int d = f / 2;
+  ST q[5], m[3];
+#pragma unroll
+  for (int c = 0; c < 5; ++c) q[c] = Q[(long long)c * L.npad + src];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) m[c] = (ST)M[(long long)(3 * d + c) * L.npad + nb];
+  const ST sgn = (f % 2 == 0) ? ST(-1) : ST(1);
+  const ST inv = BcMath<ST, FAST>::div(sgn, BcMath<ST, FAST>::sqrt_(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]));
+  const ST n[3] = {m[0] * inv, m[1] * inv, m[2] * inv};
+  riemann_farfield<ST, FAST>(F, q, n, v);
   return true;
 }
 
-// Boundary fill in one pass over the padded nodes of the slabs (bc_slabs:
-// outside the updated box, one or two ghost layers deep), nodes [t_begin,
-// t_end) of slab q with stride t_step: each takes the value of the grid
-// node its index maps to (wrap, clamp for the ghost layers behind a face,
-// or across the centreline of a cylindrical grid): a
-// copy when that node is updated by the stages, its boundary-condition value
-// (computed here from the interior node it reads, or, on the centreline,
-// from the azimuthal means computed before this pass) when it is a boundary
-// node.  Only updated nodes are read, so the pass is race-free in one
-// launch, and every node gets the value of a boundary pass followed by a
-// ghost copy.
-template <typename ST, typename MT, bool FAST>
-__device__ __forceinline__ void fill_slab(const Layout& L, const Slabs& sl, int q, int t_begin, int t_step, int t_end,
-                                          const double* inflow,
+template <typename ST>
+__device__ __forceinline__ void put_node(const Layout& L, ST* Q, int i, int j, int k, const ST v[5]) {
+  const long long o = L.at(i, j, k);
+#pragma unroll
+  for (int c = 0; c < 5; ++c) Q[(long long)c * L.npad + o] = v[c];
+}
+
+// Boundary fill over the padded nodes of the slabs (bc_slabs: outside the
+// updated box): one thread per position of a y or z slab's face plane, which
+// sets all layers of the slab there, and per node of an x slab.  Behind a physical face (inflow, far field) the
+// layers are images of one boundary node, whose value is formed once; behind a
+// periodic face and the centreline every layer has a node of its own.  Only
+// updated nodes are read, so the pass is race-free in one launch, and every
+// node gets the value of a boundary pass followed by a ghost copy.
+// Bound by the latency of its loads and by the boundary formulas' instructions
+// (680 per node when every layer formed its own value), not by DRAM.
+template <typename ST, typename MT, bool FAST, bool AXIS_IN>
+__device__ __forceinline__ void fill_line(const Layout& L, const Slabs& sl, int q, int p, const double* inflow,
                                           const double* axis, const FlowC& F, ST* __restrict__ Q,
                                           const MT* __restrict__ M) {
-  // one node per thread (four per thread with their loads issued together
-  // measured slower: fewer resident threads)
-  constexpr int U = 1;
-  const int tot = min(t_end, sl.e[q][0] * sl.e[q][1] * sl.e[q][2]);
-  const int bw = t_step;
-  for (int tb = t_begin; tb < tot; tb += t_step * U) {
-    long long dst[U], src[U], nb[U];
-    int kind[U], face[U], inf[U];  // kind: 0 copy, 1 inflow, 2 far field, 3 centreline, -1 none
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      int i, j, k;
-      kind[u] = -1;
-      face[u] = 0;
-      inf[u] = 0;
-      src[u] = nb[u] = dst[u] = 0;
-      if (!slab_node(sl, q, tb + u * bw, i, j, k)) continue;
-      // ghosts behind a face inside a larger grid are the halo exchange's
-      if ((i < 0 && L.bc[0] == BC_EXCHANGE) || (i >= L.n[0] && L.bc[1] == BC_EXCHANGE) ||
-          (j < 0 && L.bc[2] == BC_EXCHANGE) || (j >= L.n[1] && L.bc[3] == BC_EXCHANGE) ||
-          (k < 0 && L.bc[4] == BC_EXCHANGE) || (k >= L.n[2] && L.bc[5] == BC_EXCHANGE))
-        continue;
-      dst[u] = L.at(i, j, k);
-      int mi = i, mj = j, mk = k;
-      L.map_node(mi, mj, mk);
-      if (mi >= L.lo[0] && mi <= L.hi[0] && mj >= L.lo[1] && mj <= L.hi[1] && mk >= L.lo[2] && mk <= L.hi[2]) {
-        kind[u] = 0;
-        src[u] = L.at(mi, mj, mk);
-        continue;
-      }
-      // boundary node (mi, mj, mk): the face latest in the order y-, y+, z-,
-      // z+, x+, x- decides
-      const int idx[3] = {mi, mj, mk};
-      const int order[6] = {2, 3, 4, 5, 1, 0};
-      int f = -1;
-#pragma unroll
-      for (int o = 0; o < 6; ++o) {
-        const int ff = order[o], d = ff / 2;
-        if (L.bc[ff] == BC_PERIODIC || L.bc[ff] == BC_EXCHANGE) continue;
-        if (idx[d] == ((ff % 2 == 0) ? 0 : L.n[d] - 1)) f = ff;
-      }
-      face[u] = f;
-      if (f < 0) continue;  // not reached: a node outside the updated box lies on some face
-      if (L.bc[f] == BC_INFLOW) {  // x- face only: profile tabulated per (j, k)
-        kind[u] = 1;
-        inf[u] = mk * L.n[1] + mj;
-        continue;
-      }
-      if (L.bc[f] == BC_AXIS) {  // azimuthal mean of the adjacent radial line
-        kind[u] = 3;
-        inf[u] = mi;
-        continue;
-      }
-      kind[u] = 2;  // far field: nearest updated node, normal at the boundary node
-      int ci[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) ci[d] = idx[d] < L.lo[d] ? L.lo[d] : (idx[d] > L.hi[d] ? L.hi[d] : idx[d]);
-      src[u] = L.at(ci[0], ci[1], ci[2]);
-      // on the centreline the face metric vanishes: normal of the adjacent radial node
-      nb[u] = L.at(mi, (L.cyl && mj == 0) ? 1 : mj, mk);
-    }
-    ST qv[U][5], mv[U][3];
-    double uin[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      uin[u] = 0.0;
-      if (kind[u] == 0 || kind[u] == 2) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) qv[u][v] = Q[(long long)v * L.npad + src[u]];
-      }
-      if (kind[u] == 2) {
-        const int d = face[u] / 2;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) mv[u][c] = (ST)M[(long long)(3 * d + c) * L.npad + nb[u]];
-      }
-      if (kind[u] == 1) uin[u] = inflow[inf[u]];
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (kind[u] < 0) continue;
-      ST v[5];
-      if (kind[u] == 0) {
-#pragma unroll
-        for (int c = 0; c < 5; ++c) v[c] = qv[u][c];
-      } else if (kind[u] == 1) {
-        to_conserved<ST, FAST>(flow_const<ST>(F.gm1, F.gm1_f), ST(1), (ST)uin[u], ST(0), ST(0),
-                               flow_const<ST>(1.0 / F.gamma, F.pe_f), v);
-      } else if (kind[u] == 3) {
-#pragma unroll
-        for (int c = 0; c < 5; ++c) v[c] = (ST)axis[c * L.n[0] + inf[u]];
-      } else {
-        const ST a = mv[u][0], b = mv[u][1], cc = mv[u][2];
-        const ST sgn = (face[u] % 2 == 0) ? ST(-1) : ST(1);
-        const ST inv = BcMath<ST, FAST>::div(sgn, BcMath<ST, FAST>::sqrt_(a * a + b * b + cc * cc));
-        const ST n[3] = {a * inv, b * inv, cc * inv};
-        riemann_farfield<ST, FAST>(F, qv[u], n, v);
-      }
-#pragma unroll
-      for (int c = 0; c < 5; ++c) Q[(long long)c * L.npad + dst[u]] = v[c];
-    }
+  const int d = q < 2 ? 2 : (q < 4 ? 1 : 0);
+  const int y = p / sl.e[q][0], i = sl.a[q][0] + p - y * sl.e[q][0];
+  int j = sl.a[q][1] + y, k = sl.a[q][2] + y, l = 0, n = 1;
+  if (d == 0) {  // one node per thread: a row's layers are neighbours in memory and are stored together
+    const int z = y / sl.e[q][1];
+    j -= z * sl.e[q][1];
+    k = sl.a[q][2] + z;
+  } else {
+    l = sl.a[q][d];
+    n = sl.e[q][d];
+  }
+  const int face = 2 * d + (q & 1);
+  const bool images = L.bc[face] == BC_INFLOW || L.bc[face] == BC_FARFIELD;
+  bool set = false;
+  ST v[5];
+#pragma unroll 1
+  for (int r = 0; r < n; ++r) {
+    const int jj = d == 1 ? l + r : j, kk = d == 2 ? l + r : k;
+    if (r == 0 || !images) set = node_value<ST, MT, FAST, AXIS_IN>(L, inflow, axis, F, Q, M, i, jj, kk, v);
+    if (set) put_node(L, Q, i, jj, kk, v);
   }
 }
 
-template <typename ST, typename MT, bool FAST>
-__global__ void k_bc_fill(const __grid_constant__ Layout L, const __grid_constant__ Slabs sl,
-                          const double* __restrict__ inflow, const double* __restrict__ axis,
-                          const __grid_constant__ FlowC F, ST* __restrict__ Q, const MT* __restrict__ M) {
-  fill_slab<ST, MT, FAST>(L, sl, blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, INT_MAX, inflow,
-                    axis, F, Q, M);
+// threads of slab q: its face plane's positions, or all nodes of an x slab
+__host__ __device__ __forceinline__ int slab_positions(const Slabs& sl, int q) {
+  if (sl.e[q][q < 2 ? 2 : (q < 4 ? 1 : 0)] <= 0) return 0;
+  return sl.e[q][0] * (q < 4 ? 1 : sl.e[q][1]) * (q < 2 ? sl.e[q][1] : sl.e[q][2]);
 }
+
+// blocks of one launch: the centreline means' (FP32 cylinders), then the slabs'
+struct FillBlocks {
+  int axis, first[7];  // first block of every slab; first[6]: all
+};
 
 // Centreline of a cylindrical grid (the paper's singularity treatment,
 // Section 3 and Section 4.3): for every axial index i and variable v, the
@@ -427,7 +412,7 @@ __global__ void k_bc_fill(const __grid_constant__ Layout L, const __grid_constan
 // parallel, the azimuth going through shared memory in chunks of 24 KB (96
 // FP64 values per i), seven warps loading the next chunk (one coalesced row
 // of 32 i per load) while warp 0 adds the current one value by value in
-// azimuthal order.  FP32 states take axis_mean_f32 below.
+// azimuthal order.  FP32 states take axis_block below.
 constexpr int AX_WARPS = 8;
 constexpr int AX_BYTES = 24576;  // one chunk buffer; two are used
 
@@ -487,88 +472,124 @@ __device__ __forceinline__ void axis_mean(const Layout& L, const ST* __restrict_
 // non-finite values, warp 0 runs the sequential chain.  On GB300 a warp-wide
 // FP64 add or conversion occupies the FP64 pipe for many cycles, so the
 // chain of P of them took about 30 us per launch on its own.
-__device__ __forceinline__ void axis_mean_f32(const Layout& L, const float* __restrict__ Q, double* __restrict__ axis) {
+// One block takes 32 consecutive i (from 32 ib, lane = i) of variable v, holds
+// up to 48 azimuthal values per thread in registers (all loads in flight at
+// once, one read for both passes: 13.7 us with twelve at a time and two reads)
+// and writes the centreline nodes and their azimuthal ghosts itself, so it is
+// part of the boundary pass.
+__device__ __forceinline__ void axis_block(const Layout& L, float* Q, int ib, int v) {
+  constexpr int KR = 48;
   __shared__ int s_emin[AX_WARPS][32];
   __shared__ float s_abs[AX_WARPS][32];
   __shared__ long long s_acc[AX_WARPS][32];
   __shared__ int s_exact[32];
+  __shared__ float s_mean[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int v = blockIdx.y, P = L.pn[2];
-  for (int bx = blockIdx.x; bx * 32 < L.n[0]; bx += gridDim.x) {  // block-uniform trip count
-    const int i = bx * 32 + lane;
-    const bool live = i < L.n[0];
-    const float* q = Q + (long long)v * L.npad + L.at(live ? i : 0, 1, 0);
-    int emin = INT_MAX;  // exponent of the smallest unit in the last place (nonzero values)
-    float sabs = 0.f;    // sum of magnitudes; +inf marks a non-finite value
-    if (live) {
-#pragma unroll 12
-      for (int k = w; k < P; k += AX_WARPS) {
-        const unsigned b = __float_as_uint(q[(long long)k * L.plane]);
-        const int E = (int)((b >> 23) & 0xffu);
-        if (E == 255) sabs = INFINITY;
-        if ((b & 0x7fffffffu) != 0u) emin = min(emin, E == 0 ? -149 : E - 150);
-        sabs += __uint_as_float(b & 0x7fffffffu);
-      }
+  const int P = L.pn[2], i = ib * 32 + lane;
+  const bool live = i >= L.lo[0] && i <= L.hi[0];
+  float* const Qv = Q + (long long)v * L.npad;
+  const float* q = Qv + L.at(live ? i : L.lo[0], 1, 0);
+  float x[KR];
+  auto load = [&](int base) {
+#pragma unroll
+    for (int r = 0; r < KR; ++r) {
+      const int k = base + w + r * AX_WARPS;
+      x[r] = k < P ? q[(long long)k * L.plane] : 0.f;
     }
-    s_emin[w][lane] = emin;
-    s_abs[w][lane] = sabs;
-    __syncthreads();
-    if (w == 0) {
-      int em = INT_MAX;
-      float sa = 0.f;
-      for (int r = 0; r < AX_WARPS; ++r) {
-        em = min(em, s_emin[r][lane]);
-        sa += s_abs[r][lane];
-      }
-      // the FP32 sum of P magnitudes is within a factor 1 + 2 P 2^-24 of the true sum
-      const bool exact = em == INT_MAX ||
-                         (isfinite(sa) && (double)sa * (1.0 + 2.0 * P * 0x1p-24) < ldexp(1.0, em + 53));
-      s_exact[lane] = exact;
-      s_emin[0][lane] = em;
+  };
+  int emin = INT_MAX;  // exponent of the smallest unit in the last place (nonzero values)
+  float sabs = 0.f;    // sum of magnitudes; +inf marks a non-finite value
+  for (int base = 0; base < P; base += KR * AX_WARPS) {
+    load(base);
+#pragma unroll
+    for (int r = 0; r < KR; ++r) {
+      const unsigned b = __float_as_uint(x[r]);
+      const int E = (int)((b >> 23) & 0xffu);
+      if (E == 255) sabs = INFINITY;
+      if ((b & 0x7fffffffu) != 0u) emin = min(emin, E == 0 ? -149 : E - 150);
+      sabs += __uint_as_float(b & 0x7fffffffu);
     }
-    __syncthreads();
-    const int em = s_emin[0][lane];
-    const bool exact = s_exact[lane] != 0;
-    long long acc = 0;
-    if (live && exact && em != INT_MAX) {
-#pragma unroll 12
-      for (int k = w; k < P; k += AX_WARPS) {
-        const unsigned b = __float_as_uint(q[(long long)k * L.plane]);
+  }
+  s_emin[w][lane] = emin;
+  s_abs[w][lane] = sabs;
+  __syncthreads();
+  if (w == 0) {
+    int em = INT_MAX;
+    float sa = 0.f;
+    for (int r = 0; r < AX_WARPS; ++r) {
+      em = min(em, s_emin[r][lane]);
+      sa += s_abs[r][lane];
+    }
+    // the FP32 sum of P magnitudes is within a factor 1 + 2 P 2^-24 of the true sum
+    s_exact[lane] =
+        em == INT_MAX || (isfinite(sa) && (double)sa * (1.0 + 2.0 * P * 0x1p-24) < ldexp(1.0, em + 53));
+    s_emin[0][lane] = em;
+  }
+  __syncthreads();
+  const int em = s_emin[0][lane];
+  const bool exact = s_exact[lane] != 0;
+  long long acc = 0;
+  if (exact && em != INT_MAX) {
+    for (int base = 0; base < P; base += KR * AX_WARPS) {
+      if (P > KR * AX_WARPS) load(base);
+#pragma unroll
+      for (int r = 0; r < KR; ++r) {
+        const unsigned b = __float_as_uint(x[r]);
         const int E = (int)((b >> 23) & 0xffu);
         const long long m = (long long)((b & 0x7fffffu) | (E ? 0x800000u : 0u));
-        const long long t = m << ((E == 0 ? -149 : E - 150) - em);  // < 2^53 by the bound
+        const long long t = m ? m << ((E == 0 ? -149 : E - 150) - em) : 0;  // < 2^53 by the bound
         acc += (b >> 31) ? -t : t;
       }
     }
-    s_acc[w][lane] = acc;
-    __syncthreads();
-    if (w == 0 && live) {
-      double s = 0.0;
-      if (exact) {
-        long long t = 0;
-        for (int r = 0; r < AX_WARPS; ++r) t += s_acc[r][lane];
-        s = em == INT_MAX ? 0.0 : ldexp((double)t, em);
-      } else {
-        for (int k = 0; k < P; ++k) s += (double)q[(long long)k * L.plane];
-      }
-      axis[v * L.n[0] + i] = s / P;
-    }
-    __syncthreads();  // the shared arrays are reused by the next 32 columns
   }
+  s_acc[w][lane] = acc;
+  __syncthreads();
+  if (w == 0) {
+    double s = 0.0;
+    if (exact) {
+      long long t = 0;
+      for (int r = 0; r < AX_WARPS; ++r) t += s_acc[r][lane];
+      s = em == INT_MAX ? 0.0 : ldexp((double)t, em);
+    } else {
+      for (int k = 0; k < P; ++k) s += (double)q[(long long)k * L.plane];
+    }
+    s_mean[lane] = (float)(s / P);
+  }
+  __syncthreads();
+  if (live)
+    for (int k = w - NG; k < L.n[2] + NG; k += AX_WARPS) Qv[L.at(i, 0, k)] = s_mean[lane];
 }
 
-template <typename ST>
-__device__ __forceinline__ void axis_mean_any(const Layout& L, const ST* __restrict__ Q, double* __restrict__ axis) {
-  if constexpr (sizeof(ST) == 4)
-    axis_mean_f32(L, Q, axis);
-  else
-    axis_mean<ST>(L, Q, axis);
-}
-
-template <typename ST>
-__global__ void __launch_bounds__(32 * AX_WARPS) k_axis_mean(const __grid_constant__ Layout L, const ST* __restrict__ Q,
+// FP64 states: the means into the grid's axis table, before the boundary pass
+__global__ void __launch_bounds__(32 * AX_WARPS) k_axis_mean(const __grid_constant__ Layout L, const double* __restrict__ Q,
                                                              double* __restrict__ axis) {
-  axis_mean_any<ST>(L, Q, axis);
+  axis_mean<double>(L, Q, axis);
+}
+
+// threads of a boundary-pass block: small blocks spread the FP64 formulas over
+// the SMs' narrow FP64 pipes; a centreline mean takes AX_WARPS warps
+template <typename ST, bool CYL>
+constexpr int fill_threads() { return sizeof(ST) == 8 ? 64 : (CYL ? 32 * AX_WARPS : 128); }
+
+template <typename ST, typename MT, bool FAST, bool CYL>
+__global__ void __launch_bounds__(fill_threads<ST, CYL>(), CYL ? 3 : 1)
+    k_bc_fill(const __grid_constant__ Layout L, const __grid_constant__ Slabs sl, const __grid_constant__ FillBlocks fb,
+              const double* __restrict__ inflow, const double* __restrict__ axis, const __grid_constant__ FlowC F,
+              ST* __restrict__ Q, const MT* __restrict__ M) {
+  constexpr bool AXIS_IN = CYL && sizeof(ST) == 4;
+  int b = blockIdx.x;
+  if constexpr (AXIS_IN) {
+    if (b < fb.axis) {
+      axis_block(L, Q, b / 5, b % 5);
+      return;
+    }
+    b -= fb.axis;
+  }
+  int q = 0;
+#pragma unroll
+  for (int r = 1; r < 6; ++r) q += b >= fb.first[r];
+  const int p = (b - fb.first[q]) * (int)blockDim.x + threadIdx.x;
+  if (p < slab_positions(sl, q)) fill_line<ST, MT, FAST, AXIS_IN>(L, sl, q, p, inflow, axis, F, Q, M);
 }
 
 // batched versions: grid blockIdx.z of the table, state copy `which`
@@ -582,21 +603,29 @@ struct BcCtx {
   const void* M;
 };
 
-// one work item per block: (grid, slab, first node, end node) of the slab's
-// enumeration, at most BC_ITEM_NODES nodes, so that the blocks follow the
-// slab sizes of uneven grids
-template <typename ST, typename MT, bool FAST>
-__global__ void k_bc_fill_batch(const BcCtx* __restrict__ ctx, const int4* __restrict__ items, int which) {
+// one work item per block: (grid, slab, first position, end position) of the
+// slab's face plane, at most BC_ITEM positions, so that the blocks follow the
+// slab sizes of uneven grids; slab 6: centreline means (grid, 6, i-block,
+// variable) of an FP32 cylinder
+template <typename ST, typename MT, bool FAST, bool CYL>
+__global__ void __launch_bounds__(32 * AX_WARPS)
+    k_bc_fill_batch(const BcCtx* __restrict__ ctx, const int4* __restrict__ items, int which) {
+  constexpr bool AXIS_IN = CYL && sizeof(ST) == 4;
   const int4 w = items[blockIdx.x];
   const BcCtx& X = ctx[w.x];
-  fill_slab<ST, MT, FAST>(X.L, X.fill, w.y, w.z + threadIdx.x, blockDim.x, w.w, X.inflow, X.axis, X.F, (ST*)X.Q[which],
-                    (const MT*)X.M);
+  if constexpr (AXIS_IN) {
+    if (w.y == 6) {
+      axis_block(X.L, (float*)X.Q[which], w.z, w.w);
+      return;
+    }
+  }
+  for (int p = w.z + threadIdx.x; p < w.w; p += blockDim.x)
+    fill_line<ST, MT, FAST, AXIS_IN>(X.L, X.fill, w.y, p, X.inflow, X.axis, X.F, (ST*)X.Q[which], (const MT*)X.M);
 }
 
-template <typename ST>
 __global__ void __launch_bounds__(32 * AX_WARPS) k_axis_mean_batch(const BcCtx* __restrict__ ctx, int which) {
   const BcCtx& X = ctx[blockIdx.z];
-  if (X.L.cyl) axis_mean_any<ST>(X.L, (const ST*)X.Q[which], X.axis);
+  if (X.L.cyl) axis_mean<double>(X.L, (const double*)X.Q[which], X.axis);
 }
 
 // Halo exchange between blocks of one grid (the paper's ghost exchange,
@@ -838,46 +867,39 @@ Slabs bc_slabs(const Layout& L, bool full) {
   return make_slabs(pad_lo, pad_hi, L.lo, L.hi);
 }
 
-// blocks per slab: at most 128 (six slabs then hold about one resident wave
-// of the fill's 256-thread blocks, which stride over their slab; on the
-// 256x192x192 grid 0.031 ms per fill against 0.036 ms with up to 1024)
-int slab_blocks(const Slabs& sl) {
-  long long big = 1;
-  for (int q = 0; q < 6; ++q) {
-    long long c = (long long)sl.e[q][0] * sl.e[q][1] * sl.e[q][2];
-    big = c > big ? c : big;
-  }
-  int b = grid_blocks(big, 256);
-  return b < 128 ? b : 128;
+template <typename ST, typename MT, bool FAST, bool CYL>
+static void launch_fill(const GridDev& g, const Slabs& sl, void* Q, cudaStream_t s) {
+  constexpr int T = fill_threads<ST, CYL>();
+  FillBlocks fb;
+  fb.axis = CYL && sizeof(ST) == 4 ? 5 * ((g.L.n[0] + 31) / 32) : 0;
+  fb.first[0] = 0;
+  for (int q = 0; q < 6; ++q) fb.first[q + 1] = fb.first[q] + (slab_positions(sl, q) + T - 1) / T;
+  k_bc_fill<ST, MT, FAST, CYL><<<fb.axis + fb.first[6], T, 0, s>>>(g.L, sl, fb, g.inflow, g.axis, g.F, (ST*)Q,
+                                                                   (const MT*)g.M);
+  count_launches(1);
 }
 
 cudaError_t launch_bc(const GridDev& g, void* Q, cudaStream_t s, bool full) {
   const Slabs sl = bc_slabs(g.L, full);
-  const dim3 b(slab_blocks(sl), 6);
-  if (g.L.cyl) {
-    const dim3 ab((g.L.n[0] + 31) / 32, 5);
-    if (g.prec == JZ_P64)
-      k_axis_mean<double><<<ab, 32 * AX_WARPS, 0, s>>>(g.L, (const double*)Q, g.axis);
-    else
-      k_axis_mean<float><<<ab, 32 * AX_WARPS, 0, s>>>(g.L, (const float*)Q, g.axis);
+  if (g.L.cyl && g.prec == JZ_P64) {
+    k_axis_mean<<<dim3((g.L.n[0] + 31) / 32, 5), 32 * AX_WARPS, 0, s>>>(g.L, (const double*)Q, g.axis);
     count_launches(1);
   }
   switch (g.prec) {
-    case JZ_P64:
-      k_bc_fill<double, double, false><<<b, 256, 0, s>>>(g.L, sl, g.inflow, g.axis, g.F, (double*)Q,
-                                                         (const double*)g.M);
-      break;
+    case JZ_P64: launch_fill<double, double, false, false>(g, sl, Q, s); break;
     case JZ_P32_M64:
-      k_bc_fill<float, double, true><<<b, 256, 0, s>>>(g.L, sl, g.inflow, g.axis, g.F, (float*)Q, (const double*)g.M);
+      if (g.L.cyl) launch_fill<float, double, true, true>(g, sl, Q, s);
+      else launch_fill<float, double, true, false>(g, sl, Q, s);
       break;
     case JZ_P32_S64:
-      k_bc_fill<float, float, false><<<b, 256, 0, s>>>(g.L, sl, g.inflow, g.axis, g.F, (float*)Q, (const float*)g.M);
+      if (g.L.cyl) launch_fill<float, float, false, true>(g, sl, Q, s);
+      else launch_fill<float, float, false, false>(g, sl, Q, s);
       break;
     default:
-      k_bc_fill<float, float, true><<<b, 256, 0, s>>>(g.L, sl, g.inflow, g.axis, g.F, (float*)Q, (const float*)g.M);
+      if (g.L.cyl) launch_fill<float, float, true, true>(g, sl, Q, s);
+      else launch_fill<float, float, true, false>(g, sl, Q, s);
       break;
   }
-  count_launches(1);
   return cudaGetLastError();
 }
 
@@ -899,30 +921,38 @@ void bc_ctx_fill(void* dst, const GridDev& g) {
 
 void bc_fill_items(const GridDev& g, int grid, std::vector<int4>& out) {
   const Slabs sl = bc_slabs(g.L, false);
+  if (g.L.cyl && g.prec != JZ_P64)
+    for (int ib = 0; ib * 32 < g.L.n[0]; ++ib)
+      for (int v = 0; v < 5; ++v) out.push_back(make_int4(grid, 6, ib, v));
   for (int q = 0; q < 6; ++q) {
-    const int tot = sl.e[q][0] * sl.e[q][1] * sl.e[q][2];
-    for (int t = 0; t < tot; t += BC_ITEM_NODES) out.push_back(make_int4(grid, q, t, std::min(tot, t + BC_ITEM_NODES)));
+    const int tot = slab_positions(sl, q);
+    for (int t = 0; t < tot; t += BC_ITEM) out.push_back(make_int4(grid, q, t, std::min(tot, t + BC_ITEM)));
   }
 }
 
+template <typename ST, typename MT, bool FAST>
+static void launch_fill_batch(const BcCtx* X, const int4* items, int nitems, int which, bool cyl, cudaStream_t s) {
+  if (cyl && sizeof(ST) == 4)
+    k_bc_fill_batch<ST, MT, FAST, true><<<nitems, 32 * AX_WARPS, 0, s>>>(X, items, which);
+  else
+    k_bc_fill_batch<ST, MT, FAST, false><<<nitems, fill_threads<ST, false>(), 0, s>>>(X, items, which);
+  count_launches(1);
+}
+
+// cyl: some grid of the batch is cylindrical
 cudaError_t launch_bc_batch(int prec, const void* ctx, int n, const int4* items, int nitems, int which, bool cyl,
                             cudaStream_t s) {
   const BcCtx* X = (const BcCtx*)ctx;
-  if (cyl) {  // some grid of the batch is cylindrical: centreline means first
-    const dim3 ab(8, 5, n);
-    if (prec == JZ_P64)
-      k_axis_mean_batch<double><<<ab, 32 * AX_WARPS, 0, s>>>(X, which);
-    else
-      k_axis_mean_batch<float><<<ab, 32 * AX_WARPS, 0, s>>>(X, which);
+  if (cyl && prec == JZ_P64) {  // centreline means first
+    k_axis_mean_batch<<<dim3(8, 5, n), 32 * AX_WARPS, 0, s>>>(X, which);
     count_launches(1);
   }
   switch (prec) {
-    case JZ_P64: k_bc_fill_batch<double, double, false><<<nitems, 256, 0, s>>>(X, items, which); break;
-    case JZ_P32_M64: k_bc_fill_batch<float, double, true><<<nitems, 256, 0, s>>>(X, items, which); break;
-    case JZ_P32_S64: k_bc_fill_batch<float, float, false><<<nitems, 256, 0, s>>>(X, items, which); break;
-    default: k_bc_fill_batch<float, float, true><<<nitems, 256, 0, s>>>(X, items, which); break;
+    case JZ_P64: launch_fill_batch<double, double, false>(X, items, nitems, which, cyl, s); break;
+    case JZ_P32_M64: launch_fill_batch<float, double, true>(X, items, nitems, which, cyl, s); break;
+    case JZ_P32_S64: launch_fill_batch<float, float, false>(X, items, nitems, which, cyl, s); break;
+    default: launch_fill_batch<float, float, true>(X, items, nitems, which, cyl, s); break;
   }
-  count_launches(1);
   return cudaGetLastError();
 }
 

@@ -73,9 +73,9 @@ cudaError_t launch_pack_metric(const GridDev& g, int f, double* dense, cudaStrea
 // batched boundary fill over a device table of per-grid contexts
 size_t bc_ctx_bytes();
 void bc_ctx_fill(void* host_dst, const GridDev& g);
-// batched boundary pass: work items (grid, slab, first node, end node) of at
-// most BC_ITEM_NODES nodes (one 256-thread block each)
-constexpr int BC_ITEM_NODES = 1024;
+// batched boundary pass: work items (grid, slab, first position, end position)
+// of at most BC_ITEM positions of a slab's face plane (one block each)
+constexpr int BC_ITEM = 256;
 void bc_fill_items(const GridDev& g, int grid, std::vector<int4>& out);
 cudaError_t launch_bc_batch(int prec, const void* ctx, int n, const int4* items, int nitems, int which, bool cyl,
                             cudaStream_t s);
