@@ -400,6 +400,7 @@ __host__ __device__ __forceinline__ int slab_positions(const Slabs& sl, int q) {
 // blocks of one launch: the centreline means' (FP32 cylinders), then the slabs'
 struct FillBlocks {
   int axis, first[7];  // first block of every slab; first[6]: all
+  int one_wave;        // the blocks are resident together
 };
 
 // Centreline of a cylindrical grid (the paper's singularity treatment,
@@ -577,6 +578,8 @@ __global__ void __launch_bounds__(fill_threads<ST, CYL>(), CYL ? 3 : 1)
               const double* __restrict__ inflow, const double* __restrict__ axis, const __grid_constant__ FlowC F,
               ST* __restrict__ Q, const MT* __restrict__ M) {
   constexpr bool AXIS_IN = CYL && sizeof(ST) == 4;
+  if (fb.one_wave) let_next_start();
+  wait_for_previous();
   int b = blockIdx.x;
   if constexpr (AXIS_IN) {
     if (b < fb.axis) {
@@ -868,15 +871,16 @@ Slabs bc_slabs(const Layout& L, bool full) {
 }
 
 template <typename ST, typename MT, bool FAST, bool CYL>
-static void launch_fill(const GridDev& g, const Slabs& sl, void* Q, cudaStream_t s) {
+static cudaError_t launch_fill(const GridDev& g, const Slabs& sl, void* Q, cudaStream_t s) {
   constexpr int T = fill_threads<ST, CYL>();
   FillBlocks fb;
   fb.axis = CYL && sizeof(ST) == 4 ? 5 * ((g.L.n[0] + 31) / 32) : 0;
   fb.first[0] = 0;
   for (int q = 0; q < 6; ++q) fb.first[q + 1] = fb.first[q] + (slab_positions(sl, q) + T - 1) / T;
-  k_bc_fill<ST, MT, FAST, CYL><<<fb.axis + fb.first[6], T, 0, s>>>(g.L, sl, fb, g.inflow, g.axis, g.F, (ST*)Q,
-                                                                   (const MT*)g.M);
+  fb.one_wave = fb.axis + fb.first[6] <= 8 * device_sm_count();
   count_launches(1);
+  return launch_dep(k_bc_fill<ST, MT, FAST, CYL>, dim3(fb.axis + fb.first[6]), T, 0, s, g.L, sl, fb, g.inflow, g.axis, g.F,
+                    (ST*)Q, (const MT*)g.M);
 }
 
 cudaError_t launch_bc(const GridDev& g, void* Q, cudaStream_t s, bool full) {
@@ -886,21 +890,17 @@ cudaError_t launch_bc(const GridDev& g, void* Q, cudaStream_t s, bool full) {
     count_launches(1);
   }
   switch (g.prec) {
-    case JZ_P64: launch_fill<double, double, false, false>(g, sl, Q, s); break;
+    case JZ_P64: return launch_fill<double, double, false, false>(g, sl, Q, s);
     case JZ_P32_M64:
-      if (g.L.cyl) launch_fill<float, double, true, true>(g, sl, Q, s);
-      else launch_fill<float, double, true, false>(g, sl, Q, s);
-      break;
+      return g.L.cyl ? launch_fill<float, double, true, true>(g, sl, Q, s)
+                     : launch_fill<float, double, true, false>(g, sl, Q, s);
     case JZ_P32_S64:
-      if (g.L.cyl) launch_fill<float, float, false, true>(g, sl, Q, s);
-      else launch_fill<float, float, false, false>(g, sl, Q, s);
-      break;
+      return g.L.cyl ? launch_fill<float, float, false, true>(g, sl, Q, s)
+                     : launch_fill<float, float, false, false>(g, sl, Q, s);
     default:
-      if (g.L.cyl) launch_fill<float, float, true, true>(g, sl, Q, s);
-      else launch_fill<float, float, true, false>(g, sl, Q, s);
-      break;
+      return g.L.cyl ? launch_fill<float, float, true, true>(g, sl, Q, s)
+                     : launch_fill<float, float, true, false>(g, sl, Q, s);
   }
-  return cudaGetLastError();
 }
 
 size_t bc_ctx_bytes() { return sizeof(BcCtx); }

@@ -226,6 +226,7 @@ __device__ __forceinline__ void timestep_body(const Layout& L, const FlowC& F, c
       }
     }
   }
+  let_next_start();  // no effect in the batched kernel
   double best = (double)best_s;
   __shared__ double red[RED_THREADS / 32];
   best = warp_max(best);
@@ -272,6 +273,7 @@ template <typename ST, typename MT, bool DIAG = false>
 __global__ void __launch_bounds__(RED_THREADS) k_timestep(Layout L, FlowC F, const ST* __restrict__ Q,
                                                           const MT* __restrict__ M, Scalars* sc, double* partial,
                                                           double cfl, bool finalize) {
+  wait_for_previous();
   timestep_body<ST, MT, DIAG>(L, F, Q, M, sc, partial, cfl, finalize);
 }
 
@@ -365,6 +367,23 @@ __global__ void __launch_bounds__(RED_THREADS) k_diag(Layout L, FlowC F, const S
 
 }  // namespace
 
+template <bool DIAG>
+static cudaError_t launch_reduction(const GridDev& g, double cfl, bool finalize, cudaStream_t s) {
+  const int nb = red_grid(2);
+  count_launches(1);
+  switch (g.prec) {
+    case JZ_P64:
+      return launch_dep(k_timestep<double, double, DIAG>, dim3(nb), RED_THREADS, 0, s, g.L, g.F, (const double*)g.Q0,
+                        (const double*)g.M, g.sc, g.partial, cfl, finalize);
+    case JZ_P32_M64:
+      return launch_dep(k_timestep<float, double, DIAG>, dim3(nb), RED_THREADS, 0, s, g.L, g.F, (const float*)g.Q0,
+                        (const double*)g.M, g.sc, g.partial, cfl, finalize);
+    default:
+      return launch_dep(k_timestep<float, float, DIAG>, dim3(nb), RED_THREADS, 0, s, g.L, g.F, (const float*)g.Q0,
+                        (const float*)g.M, g.sc, g.partial, cfl, finalize);
+  }
+}
+
 cudaError_t launch_timestep(const GridDev& g, double cfl, double dt_fixed, cudaStream_t s) {
   if (cfl <= 0.0) {
     if (g.step_diag) {  // the diagnostics of the step's state by their own pass
@@ -375,61 +394,10 @@ cudaError_t launch_timestep(const GridDev& g, double cfl, double dt_fixed, cudaS
     count_launches(1);
     return cudaGetLastError();
   }
-  const int nb = red_grid(2);
-  if (g.step_diag) {
-    switch (g.prec) {
-      case JZ_P64:
-        k_timestep<double, double, true><<<nb, RED_THREADS, 0, s>>>(g.L, g.F, (const double*)g.Q0,
-                                                                   (const double*)g.M, g.sc, g.partial, cfl, true);
-        break;
-      case JZ_P32_M64:
-        k_timestep<float, double, true><<<nb, RED_THREADS, 0, s>>>(g.L, g.F, (const float*)g.Q0,
-                                                                  (const double*)g.M, g.sc, g.partial, cfl, true);
-        break;
-      default:
-        k_timestep<float, float, true><<<nb, RED_THREADS, 0, s>>>(g.L, g.F, (const float*)g.Q0, (const float*)g.M,
-                                                                 g.sc, g.partial, cfl, true);
-        break;
-    }
-    count_launches(1);
-    return cudaGetLastError();
-  }
-  switch (g.prec) {
-    case JZ_P64:
-      k_timestep<double, double><<<nb, RED_THREADS, 0, s>>>(g.L, g.F, (const double*)g.Q0, (const double*)g.M, g.sc,
-                                                            g.partial, cfl, true);
-      break;
-    case JZ_P32_M64:
-      k_timestep<float, double><<<nb, RED_THREADS, 0, s>>>(g.L, g.F, (const float*)g.Q0, (const double*)g.M, g.sc,
-                                                           g.partial, cfl, true);
-      break;
-    default:
-      k_timestep<float, float><<<nb, RED_THREADS, 0, s>>>(g.L, g.F, (const float*)g.Q0, (const float*)g.M, g.sc,
-                                                          g.partial, cfl, true);
-      break;
-  }
-  count_launches(1);
-  return cudaGetLastError();
+  return g.step_diag ? launch_reduction<true>(g, cfl, true, s) : launch_reduction<false>(g, cfl, true, s);
 }
 
-cudaError_t launch_rate(const GridDev& g, cudaStream_t s) {
-  switch (g.prec) {
-    case JZ_P64:
-      k_timestep<double, double><<<red_grid(2), RED_THREADS, 0, s>>>(g.L, g.F, (const double*)g.Q0,
-                                                                    (const double*)g.M, g.sc, g.partial, 1.0, false);
-      break;
-    case JZ_P32_M64:
-      k_timestep<float, double><<<red_grid(2), RED_THREADS, 0, s>>>(g.L, g.F, (const float*)g.Q0,
-                                                                   (const double*)g.M, g.sc, g.partial, 1.0, false);
-      break;
-    default:
-      k_timestep<float, float><<<red_grid(2), RED_THREADS, 0, s>>>(g.L, g.F, (const float*)g.Q0, (const float*)g.M,
-                                                                  g.sc, g.partial, 1.0, false);
-      break;
-  }
-  count_launches(1);
-  return cudaGetLastError();
-}
+cudaError_t launch_rate(const GridDev& g, cudaStream_t s) { return launch_reduction<false>(g, 1.0, false, s); }
 
 cudaError_t launch_advance_from_rate(const GridDev& g, double cfl, cudaStream_t s) {
   k_advance_from_rate<<<1, 1, 0, s>>>(g.sc, cfl);

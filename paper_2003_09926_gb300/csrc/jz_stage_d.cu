@@ -675,6 +675,7 @@ __global__ void __launch_bounds__(C::NT, C::MINB)
     k_stage_d(const __grid_constant__ StageCtx<double, double> X, const StageSel st) {
   extern __shared__ __align__(128) unsigned char smem[];
   tm_alloc<C>(smem);
+  wait_for_previous();
   if (threadIdx.x < C::NTILE)
     item_d<C, MD, 0>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true);
   else
@@ -724,9 +725,8 @@ cudaError_t launch(const StageCtx<double, double>& X, const StageSel& st, cudaSt
   const Layout& L = X.L;
   const int nz = L.hi[2] - L.lo[2] + 1;
   const dim3 grid((L.hi[0] + C::TI) / C::TI, (L.hi[1] + C::TJ) / C::TJ, (nz + X.kc - 1) / X.kc);
-  k_stage_d<C, MD><<<grid, C::NT, C::BYTES, s>>>(X, st);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_dep(k_stage_d<C, MD>, grid, C::NT, C::BYTES, s, X, st);
 }
 
 template <class C, int MD>

@@ -935,6 +935,7 @@ __global__ void __launch_bounds__(vr::NT, vr::MINB)
     k_stage_v(const __grid_constant__ StageCtx<float, float> X, const StageSel st) {
   extern __shared__ __align__(128) unsigned char smem[];
   tm_alloc(smem);
+  wait_for_previous();
   switch (role_of(threadIdx.x)) {
     case 0: item_v<MD, 0, S64>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
     case 2: item_v<MD, 2, S64>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
@@ -983,9 +984,8 @@ cudaError_t launch(const StageCtx<float, float>& X, const StageSel& st, cudaStre
   const Layout& L = X.L;
   const int nz = L.hi[2] - L.lo[2] + 1;
   dim3 grid((L.hi[0] + vr::TI) / vr::TI, (L.hi[1] + vr::TJ) / vr::TJ, (nz + X.kc - 1) / X.kc);
-  k_stage_v<MD, S64><<<grid, vr::NT, vr::BYTES, s>>>(X, st);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_dep(k_stage_v<MD, S64>, grid, vr::NT, vr::BYTES, s, X, st);
 }
 
 template <int MD, bool S64>
