@@ -12,6 +12,7 @@
 //   nu_max = max(4/3, gamma/Pr) mu(T) / rho.
 #include <cmath>
 
+#include "jz_fastmath.cuh"
 #include "jz_internal.h"
 
 namespace jz {
@@ -29,9 +30,17 @@ int red_grid(int per_sm) {
   return b < RED_BLOCKS ? b : RED_BLOCKS;
 }
 
-template <typename T>
-__device__ __forceinline__ T sutherland(T mu_inf, T s1, T temp) {
-  return mu_inf * temp * sqrt(temp) * (T(1) + s1) / (temp + s1);
+// reciprocal and square root of the reduction: IEEE in FP32 (bound by memory),
+// the short forms in FP64 (bound by the FP64 pipe)
+__device__ __forceinline__ float rd_rcp(float x) { return 1.f / x; }
+__device__ __forceinline__ double rd_rcp(double x) { return stg::rcp3(x); }
+__device__ __forceinline__ float rd_sqrt(float x) { return sqrt(x); }
+__device__ __forceinline__ double rd_sqrt(double x) { return stg::sqrt3(x); }
+__device__ __forceinline__ float sutherland(float mu_inf, float s1, float temp, float root) {
+  return mu_inf * temp * root * (1.f + s1) / (temp + s1);
+}
+__device__ __forceinline__ double sutherland(double mu_inf, double s1, double temp, double root) {
+  return mu_inf * temp * root * (1.0 + s1) * stg::rcp3(temp + s1);
 }
 
 __device__ __forceinline__ double warp_max(double v) {
@@ -167,57 +176,70 @@ __device__ __forceinline__ void timestep_body(const Layout& L, const FlowC& F, c
   // 4w + 3, then the next four after all warps, one node per lane and item,
   // with the loads of all four issued before any arithmetic (the kernel is
   // bound by memory latency; on a narrow grid the four are rows, on a wide
-  // one parts of a row).  The item counter moves as (ch, j, k) with carries:
-  // no division inside the loop.
+  // one parts of a row).  FP64 grids are bound by arithmetic instead: there
+  // the four items of a warp lie W apart, so that a small grid's items reach
+  // every SM (48x32x32: 2048 items, on 64 of 304 blocks before; 37 and 21 us).
+  // The item counter moves as (ch, j, k) with carries: no division inside the
+  // loop.
   constexpr int U = 4;
   const int lane = threadIdx.x & 31;
   const int nch = (L.n[0] + 31) >> 5;
   const long long items = (long long)L.n[1] * L.n[2] * nch;  // < 2^31, checked when the grid is created
   const int W = (gridDim.x * blockDim.x) >> 5;
-  const int first = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * U;
-  const int stride = W * U;
+  constexpr bool SPREAD = sizeof(ST) == 8;
+  const int first = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (SPREAD ? 1 : U);
+  const int step = SPREAD ? W : 1;              // between the items of a group
+  const int stride = SPREAD ? W : W * U;        // the counter's move: per item, or per group
   int ch = first % nch, j = (first / nch) % L.n[1], k = first / nch / L.n[1];
   const int dch = stride % nch, dj = (stride / nch) % L.n[1], dk = stride / nch / L.n[1];
-  for (long long it0 = first; it0 < items; it0 += stride) {
+  auto advance = [&] {
+    ch += dch;
+    j += dj;
+    k += dk;
+    if (ch >= nch) { ch -= nch; ++j; }
+    if (j >= L.n[1]) { j -= L.n[1]; ++k; }
+  };
+  for (long long it0 = first; it0 < items; it0 += (long long)W * U) {
     ST q[U][5], m[U][10];
     bool live[U];
     int cu = ch, ju = j, ku = k;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int i = cu * 32 + lane;
-      live[u] = it0 + u < items && i < L.n[0];
+      live[u] = it0 + (long long)u * step < items && i < L.n[0];
       const long long n = live[u] ? L.at(i, ju, ku) : L.at(0, 0, 0);
 #pragma unroll
       for (int v = 0; v < 5; ++v) q[u][v] = Q[v * L.npad + n];
 #pragma unroll
       for (int f = 0; f < 10; ++f) m[u][f] = (ST)M[f * L.npad + n];
-      if (++cu == nch) {
+      if (SPREAD) {
+        advance();
+        cu = ch;
+        ju = j;
+        ku = k;
+      } else if (++cu == nch) {
         cu = 0;
         if (++ju == L.n[1]) { ju = 0; ++ku; }
       }
     }
-    ch += dch;
-    j += dj;
-    k += dk;
-    if (ch >= nch) { ch -= nch; ++j; }
-    if (j >= L.n[1]) { j -= L.n[1]; ++k; }
+    if (!SPREAD) advance();
     {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (!live[u]) continue;
-        const ST rho = q[u][0], ri = ST(1) / rho;
+        const ST rho = q[u][0], ri = rd_rcp(rho);
         const ST uu = q[u][1] * ri, vv = q[u][2] * ri, ww = q[u][3] * ri;
         const ST p = gm1 * (q[u][4] - ST(0.5) * rho * (uu * uu + vv * vv + ww * ww));
         const ST T = g * p * ri;
-        const ST c = sqrt(T);
-        const ST nu = vfac * sutherland<ST>(mu_inf, s1, T) * ri;
+        const ST c = rd_sqrt(T);
+        const ST nu = vfac * sutherland(mu_inf, s1, T, c) * ri;
         const ST Jn = m[u][9];
         ST conv = 0, s2 = 0;
 #pragma unroll
         for (int kd = 0; kd < 3; ++kd) {
           const ST a = m[u][3 * kd], b = m[u][3 * kd + 1], cc = m[u][3 * kd + 2];
           const ST sq = a * a + b * b + cc * cc;
-          conv += Jn * (fabs(a * uu + b * vv + cc * ww) + c * sqrt(sq));
+          conv += Jn * (fabs(a * uu + b * vv + cc * ww) + c * rd_sqrt(sq));
           s2 += sq;
         }
         const ST rate = conv + ST(2) * nu * Jn * Jn * s2;

@@ -46,27 +46,6 @@ __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, 
 __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
 
-// 1/b: with e = 1 - b y of an approximation y, 1/b = y (1 + e + e^2 + ...);
-// |e| < 2^-20, so what is left out is below 2^-60.
-__device__ __forceinline__ double rcp3(double b) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-  const double e = fma(-b, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-
-// sqrt(x): with e = 1 - x y^2 of an approximation y to x^(-1/2) and t = x y,
-// sqrt(x) = t (1 + e/2 + 3 e^2/8 + ...); |e| < 2^-20.  Zero (tested on the bits,
-// where y is infinite) gives zero.
-__device__ __forceinline__ double sqrt3(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double t = mul(x, y);
-  const double e = fma(-t, y, 1.0);
-  const double r = fma(mul(t, e), fma(0.375, e, 0.5), t);
-  return (uint32_t)(__double2hiint(x) & 0x7fffffff) < 0x00100000u ? 0.0 : r;
-}
-
 // J^(-2/3) (of |J|): J = m 2^(3q), 1 <= m < 16; y of an FP32 approximation to
 // m^(-1/3), then with e = 1 - m y^3, m^(-1/3) = y (1 + e/3 + 2 e^2/9 + ...);
 // |e| < 2^-18, so what is left out is below 2^-56.  The exponents are integer
