@@ -246,15 +246,19 @@ __device__ void riemann_farfield(const FlowC& F, const T qi[5], const T n[3], T 
   T Rm = M::div(-T(2), gm1);  // exterior u_n = 0, c = 1
   T un = T(0.5) * (Rp + Rm);
   T c = T(0.25) * gm1 * (Rp - Rm);
-  T s, ut[3];
-  if (un > T(0)) {
-    s = M::div(p_i, M::powp(rho_i, g));
-    for (int d = 0; d < 3; ++d) ut[d] = u[d] - un_i * n[d];
+  T ut[3];
+  for (int d = 0; d < 3; ++d) ut[d] = un > T(0) ? u[d] - un_i * n[d] : T(0);
+  T rho;
+  if constexpr (sizeof(T) == 8) {
+    // with the entropy s = p/rho^g of the upwind side (rho_i, c_i or 1, 1),
+    // (c^2 / (g s))^(1/(g-1)) = rho_i (c^2 / c_i^2)^(1/(g-1)): one power
+    // instead of two (FP64 pass of 128x96x96: 62 and 37 us)
+    const T ratio = un > T(0) ? c / c_i : c;
+    rho = (un > T(0) ? rho_i : T(1)) * pow(ratio * ratio, T(1) / gm1);
   } else {
-    s = p_e;  // p_e / rho_e^g with rho_e = 1
-    for (int d = 0; d < 3; ++d) ut[d] = T(0);
+    const T s = un > T(0) ? M::div(p_i, M::powp(rho_i, g)) : p_e;
+    rho = M::powp(M::div(c * c, g * s), M::rcp(gm1));
   }
-  T rho = M::powp(M::div(c * c, g * s), M::rcp(gm1));
   T p = M::div(rho * c * c, g);
   to_conserved<T, FAST>(gm1, rho, ut[0] + un * n[0], ut[1] + un * n[1], ut[2] + un * n[2], p, qb);
 }
