@@ -221,6 +221,8 @@ struct jz_batch {
   size_t off_stage = 0, off_bc = 0, off_rate = 0, off_items = 0, off_queue = 0, off_bcitems = 0;
   int nitems = 0, nbcitems = 0;
   int model = 0;                // stage kernel flow model shared by every grid (else the runtime model)
+  bool shared = false;          // the grids' flow constants agree but for mu_inf ...
+  FlowC F;                      // ... and are these
   bool cyl = false;             // some grid is cylindrical (centreline means before each boundary pass)
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
@@ -1103,7 +1105,7 @@ int enqueue_batch_step(jz_batch* b, double cfl) {
   for (int l = 0; l < 5; ++l) {
     e = launch_stage_batch(b->prec, b->grids[0]->dev.variant, batch_tiling(b->grids[0]->dev), b->dev + b->off_stage,
                            (const int4*)(b->dev + b->off_items), b->nitems, (unsigned int*)(b->dev + b->off_queue), l,
-                           src[l], out[l], b->model, s);
+                           src[l], out[l], b->model, b->shared ? &b->F : nullptr, s);
     if (e != cudaSuccess) return fail(JZ_ECUDA, "batched stage launch failed: %s", cudaGetErrorString(e));
     e = launch_bc_batch(b->prec, b->dev + b->off_bc, n, (const int4*)(b->dev + b->off_bcitems), b->nbcitems, out[l],
                         b->cyl, s);
@@ -1160,6 +1162,9 @@ int create_batch(jz_grid* const* grids, int n, bool coupled, void* dev_buf, size
   b->model = stage_model(grids[0]->dev);
   for (int k = 1; k < n; ++k)
     if (stage_model(grids[k]->dev) != b->model) b->model = 0;  // the runtime model serves a mix
+  b->F = grids[0]->dev.F;  // as in the tables: of now
+  b->shared = true;
+  for (int k = 1; k < n; ++k) b->shared = b->shared && stage_constants_agree(grids[0]->dev.F, grids[k]->dev.F);
   b->coupled = coupled;
   b->off_x = P.off_x;
   for (int d = 0; d < 3; ++d) {

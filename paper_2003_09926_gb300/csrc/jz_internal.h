@@ -136,10 +136,13 @@ void stage_ctx_fill(void* host_dst, const GridDev& g);
 // the flow model a grid's FP32 vector-record stage kernel is compiled for
 // (the runtime model when none of the constant-flag builds matches)
 int stage_model(const GridDev& g);
-// model: the stage_model shared by every grid of the batch, else the runtime model
+// whether two grids' flow constants agree but for the viscosity mu_inf
+bool stage_constants_agree(const FlowC& a, const FlowC& b);
+// model: the stage_model shared by every grid of the batch, else the runtime
+// model; shared: flow constants that all grids agree in (but for mu_inf), else null
 cudaError_t launch_stage_batch(int prec, int variant, StageTiling tile, const void* ctx, const int4* items,
                                int nitems, unsigned int* queue, int stage, int qsel, int qout, int model,
-                               cudaStream_t s);
+                               const FlowC* shared, cudaStream_t s);
 cudaError_t stage_configure();  // one-time kernel attributes (dynamic shared memory)
 
 }  // namespace jz

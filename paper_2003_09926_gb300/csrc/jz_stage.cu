@@ -39,6 +39,7 @@
 //    workloads with constant flags and once with the flags read at run time.
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 
 #include "jz_stage_common.cuh"
 
@@ -701,17 +702,25 @@ void stage_ctx_fill(void* dst, const GridDev& g) {
   }
 }
 
+bool stage_constants_agree(const FlowC& a, const FlowC& b) {
+  KConst<float> x = make_kconst<float>(a), y = make_kconst<float>(b);
+  x.mu_inf = y.mu_inf = 0.f;
+  return memcmp(&x, &y, sizeof(x)) == 0;
+}
+
 int stage_model(const GridDev& g) { return flow_model(make_kconst<float>(g.F)); }
 
 cudaError_t launch_stage_batch(int prec, int variant, StageTiling tile, const void* ctx, const int4* items,
                                int nitems, unsigned int* queue, int stage, int qsel, int qout, int model,
-                               cudaStream_t s) {
+                               const FlowC* shared, cudaStream_t s) {
   if (variant == 2) {
     const StageSel st{kRkAlpha[stage], qsel, qout, 0};
+    const KConst<float> k = shared ? make_kconst<float>(*shared) : KConst<float>{};
+    const KConst<float>* common = shared ? &k : nullptr;
     if (prec == JZ_P32_S64) return launch_stage_v_batch_s64(ctx, items, nitems, queue, st, model, s);
-    if (tile.ti == 16 && tile.tj == 32) return launch_stage_v_batch_16x32(ctx, items, nitems, queue, st, model, s);
-    if (tile.ti == 16 && tile.tj == 16) return launch_stage_v_batch_16x16(ctx, items, nitems, queue, st, model, s);
-    return launch_stage_v_batch_32x16(ctx, items, nitems, queue, st, model, s);
+    if (tile.ti == 16 && tile.tj == 32) return launch_stage_v_batch_16x32(ctx, items, nitems, queue, st, model, common, s);
+    if (tile.ti == 16 && tile.tj == 16) return launch_stage_v_batch_16x16(ctx, items, nitems, queue, st, model, common, s);
+    return launch_stage_v_batch_32x16(ctx, items, nitems, queue, st, model, common, s);
   }
   switch (prec) {
     case JZ_P64:

@@ -251,7 +251,8 @@ constexpr int vr_ctas_per_sm(int ti, int tj) { return ti * tj <= 256 ? 2 : 1; }
   cudaError_t stage_v_configure_##S();                                                                        \
   cudaError_t launch_stage_v_##S(const stg::StageCtx<float, float>& X, const stg::StageSel& st, cudaStream_t s); \
   cudaError_t launch_stage_v_batch_##S(const void* ctx, const int4* items, int nitems, unsigned int* queue,      \
-                                       const stg::StageSel& st, int model, cudaStream_t s);
+                                       const stg::StageSel& st, int model, const stg::KConst<float>* common,    \
+                                       cudaStream_t s);
 JZ_STAGE_V_DECL(32x16)
 JZ_STAGE_V_DECL(16x32)
 JZ_STAGE_V_DECL(16x16)

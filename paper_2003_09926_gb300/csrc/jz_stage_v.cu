@@ -267,7 +267,7 @@ template <int DIR, int MD>
 __device__ __forceinline__ void node_v(const float4* __restrict__ PV, const float* __restrict__ PP,
                                        const float* __restrict__ met, int sC, const float pm5[5], const float pc5[5],
                                        const float pp5[5], float rho, float e, int x, int y, const KConst<float>& c,
-                                       float G[3][5], float lt[3], float nu[3], float& Jn) {
+                                       float mu_inf, float G[3][5], float lt[3], float nu[3], float& Jn) {
   using namespace vr;
   const int o = (y + 2) * RR + x + 2;
   const int mo = (y + 1) * RW + x + 2;
@@ -321,7 +321,7 @@ __device__ __forceinline__ void node_v(const float4* __restrict__ PV, const floa
 #pragma unroll
       for (int m = 0; m < 3; ++m) g[q][m] = hJ * (S[m] * d0[q] + S[3 + m] * d1[q] + S[6 + m] * d2[q]);
 #endif
-    const float mu = Fn<float>::div(c.mu_inf * T * Fn<float>::sqrt_(T) * c.s1p1, T + c.s1);  // Sutherland
+    const float mu = Fn<float>::div(mu_inf * T * Fn<float>::sqrt_(T) * c.s1p1, T + c.s1);  // Sutherland
     float mu_t = 0.f;
     // Smagorinsky or Vreman, Delta = J^(-1/3); an unfused product, so that
     // mu + mu_t rounds alike in the constant-flag and runtime-flag builds
@@ -506,13 +506,14 @@ __device__ __forceinline__ void widen5(const float x[5], double y[5]) {
 // update adds the FP32 increment to it in FP64, stages 1-4 round their output
 // to FP32 (it feeds only the FP32 flux evaluation), and stage 5 writes both
 // the FP64 state and its FP32 copy (the next step's flux input).
+// c: the flow constants (X.k, or those a batch's grids share), mu_inf apart.
 template <int MD, int ROLE, bool S64>
-__device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const StageSel& st, int bx, int by, int bz,
-                                       unsigned char* smem, bool first) {
+__device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const KConst<float>& c, const StageSel& st,
+                                       int bx, int by, int bz, unsigned char* smem, bool first) {
   using namespace vr;
   Smem sm(smem);
   const Layout& L = X.L;
-  const KConst<float> c = X.k;
+  const float mu_inf = X.k.mu_inf;
   const int tid = threadIdx.x;
   const int i0 = bx * TI, j0 = by * TJ;
   const int t0 = L.lo[2] + bz * X.kc;
@@ -743,7 +744,7 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
         const float* met = met_buf(t + 1);
         float G[3][5], lt[3], nu[3];
         if constexpr (ROLE == 0) {
-          node_v<0, MD>(sm.PV, sm.PP, met, sp1, pb, pt, pn, qb[0], qb[4], nx, ny, c, G, lt, nu, Jn);
+          node_v<0, MD>(sm.PV, sm.PP, met, sp1, pb, pt, pn, qb[0], qb[4], nx, ny, c, mu_inf, G, lt, nu, Jn);
 #pragma unroll
           for (int v = 0; v < 5; ++v) {
             Gi[v] = G[0][v];
@@ -753,7 +754,7 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const St
           lt3n = lt[2];
           nu3n = nu[2];
         } else if (live) {
-          node_v<ROLE, MD>(sm.PV, sm.PP, met, sp1, pb, pt, pn, qb[0], qb[4], nx, ny, c, G, lt, nu, Jn);
+          node_v<ROLE, MD>(sm.PV, sm.PP, met, sp1, pb, pt, pn, qb[0], qb[4], nx, ny, c, mu_inf, G, lt, nu, Jn);
 #pragma unroll
           for (int v = 0; v < 5; ++v) {
             if (ROLE == 1) Gi[v] = G[0][v];
@@ -952,17 +953,20 @@ __global__ void __launch_bounds__(vr::NT, vr::MINB)
   tm_alloc(smem);
   wait_for_previous();
   switch (role_of(threadIdx.x)) {
-    case 0: item_v<MD, 0, S64>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
-    case 2: item_v<MD, 2, S64>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
-    default: item_v<MD, 1, S64>(X, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
+    case 0: item_v<MD, 0, S64>(X, X.k, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
+    case 2: item_v<MD, 2, S64>(X, X.k, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
+    default: item_v<MD, 1, S64>(X, X.k, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
   }
   tm_free(smem);
 }
 
-template <int MD, bool S64>
+// SHARED: the grids agree in all flow constants but mu_inf; the constants then
+// come as a kernel parameter, whose values need no registers (from the
+// contexts they do, and the kernel spills).
+template <int MD, bool S64, bool SHARED>
 __global__ void __launch_bounds__(vr::NT, vr::MINB)
-    k_stage_v_batch(const StageCtx<float, float>* __restrict__ ctx, const int4* __restrict__ items, int nitems,
-                    unsigned int* queue, const StageSel st) {
+    k_stage_v_batch(const StageCtx<float, float>* __restrict__ ctx, const __grid_constant__ KConst<float> common,
+                    const int4* __restrict__ items, int nitems, unsigned int* queue, const StageSel st) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int next;
   bool first = true;
@@ -974,11 +978,12 @@ __global__ void __launch_bounds__(vr::NT, vr::MINB)
     __syncthreads();
     if (it >= nitems) break;
     const int4 w = items[it];
+    const KConst<float>& c = SHARED ? common : ctx[w.x].k;
     bool ok;
     switch (role_of(threadIdx.x)) {
-      case 0: ok = item_v<MD, 0, S64>(ctx[w.x], st, w.y, w.z, w.w, smem, first); break;
-      case 2: ok = item_v<MD, 2, S64>(ctx[w.x], st, w.y, w.z, w.w, smem, first); break;
-      default: ok = item_v<MD, 1, S64>(ctx[w.x], st, w.y, w.z, w.w, smem, first); break;
+      case 0: ok = item_v<MD, 0, S64>(ctx[w.x], c, st, w.y, w.z, w.w, smem, first); break;
+      case 2: ok = item_v<MD, 2, S64>(ctx[w.x], c, st, w.y, w.z, w.w, smem, first); break;
+      default: ok = item_v<MD, 1, S64>(ctx[w.x], c, st, w.y, w.z, w.w, smem, first); break;
     }
     if (!ok) break;
     first = false;
@@ -991,7 +996,9 @@ cudaError_t configure_model() {
   const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(k_stage_v<MD, S64>, at, (int)vr::BYTES);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_stage_v_batch<MD, S64>, at, (int)vr::BYTES);
+  if ((e = cudaFuncSetAttribute(k_stage_v_batch<MD, S64, false>, at, (int)vr::BYTES)) != cudaSuccess) return e;
+  if (MD != kModelSmagorinsky || S64) return e;
+  return cudaFuncSetAttribute(k_stage_v_batch<kModelSmagorinsky, false, true>, at, (int)vr::BYTES);
 }
 
 template <int MD, bool S64>
@@ -1003,14 +1010,16 @@ cudaError_t launch(const StageCtx<float, float>& X, const StageSel& st, cudaStre
   return launch_dep(k_stage_v<MD, S64>, grid, vr::NT, vr::BYTES, s, X, st);
 }
 
-template <int MD, bool S64>
+template <int MD, bool S64, bool SHARED = false>
 cudaError_t launch_batch(const void* ctx, const int4* items, int nitems, unsigned int* queue, const StageSel& st,
-                         cudaStream_t s) {
+                         cudaStream_t s, const KConst<float>* common = nullptr) {
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(unsigned int), s);
   if (e != cudaSuccess) return e;
   const int slots = device_sm_count() * vr::MINB;
   const int ctas = nitems < slots ? nitems : slots;
-  k_stage_v_batch<MD, S64><<<ctas, vr::NT, vr::BYTES, s>>>((const StageCtx<float, float>*)ctx, items, nitems, queue, st);
+  k_stage_v_batch<MD, S64, SHARED><<<ctas, vr::NT, vr::BYTES, s>>>((const StageCtx<float, float>*)ctx,
+                                                                   common ? *common : KConst<float>{}, items, nitems,
+                                                                   queue, st);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1039,11 +1048,14 @@ cudaError_t VR_FN(launch_stage_v)(const StageCtx<float, float>& X, const StageSe
 }
 
 // model: the flow model every grid of the batch shares (kModelRuntime when
-// they differ)
+// they differ); common: the flow constants they share but for mu_inf (else
+// null)
 cudaError_t VR_FN(launch_stage_v_batch)(const void* ctx, const int4* items, int nitems, unsigned int* queue,
-                                        const StageSel& st, int model, cudaStream_t s) {
+                                        const StageSel& st, int model, const KConst<float>* common, cudaStream_t s) {
   switch (model) {
-    case kModelSmagorinsky: return launch_batch<kModelSmagorinsky, false>(ctx, items, nitems, queue, st, s);
+    case kModelSmagorinsky:
+      if (common) return launch_batch<kModelSmagorinsky, false, true>(ctx, items, nitems, queue, st, s, common);
+      return launch_batch<kModelSmagorinsky, false>(ctx, items, nitems, queue, st, s);
     case kModelVreman: return launch_batch<kModelVreman, false>(ctx, items, nitems, queue, st, s);
     case kModelEuler: return launch_batch<kModelEuler, false>(ctx, items, nitems, queue, st, s);
     default: return launch_batch<kModelRuntime, false>(ctx, items, nitems, queue, st, s);
