@@ -185,6 +185,9 @@ __device__ __forceinline__ void st5j(float4* v4, float* v1, int y, int x, const 
   v4[y * vr::TI + x] = make_float4(q[0], q[1], q[2], q[3]);
   v1[y * vr::JS1 + x] = q[4];
 }
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
+}
 __device__ __forceinline__ void mbar_inval(uint64_t* bar) {
   asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
@@ -571,6 +574,7 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const KC
   // generic-proxy writes to the buffers the prologue stages into, then the barrier
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
+  if (first) wait_for_previous();
 
   // thread 0's record of its copies: bit b of pend = barrier b has had one,
   // bit b of ppar = the parity of the last one's phase
@@ -950,8 +954,12 @@ template <int MD, bool S64>
 __global__ void __launch_bounds__(vr::NT, vr::MINB)
     k_stage_v(const __grid_constant__ StageCtx<float, float> X, const StageSel st) {
   extern __shared__ __align__(128) unsigned char smem[];
+  if (threadIdx.x == 0) {  // with the barriers' set-up, before the previous kernel's results are needed
+    prefetch_map(&X.tmQ[st.qin]);
+    prefetch_map(&X.tmMv);
+    prefetch_map(&X.tmQ0u);
+  }
   tm_alloc(smem);
-  wait_for_previous();
   switch (role_of(threadIdx.x)) {
     case 0: item_v<MD, 0, S64>(X, X.k, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
     case 2: item_v<MD, 2, S64>(X, X.k, st, blockIdx.x, blockIdx.y, blockIdx.z, smem, true); break;
