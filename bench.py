@@ -140,10 +140,10 @@ def measured_hbm_peak():
 # kernel and its headers, and jz_api.cu (TMA tensor maps, default tile shape)
 STAGE_SOURCES = {2: ("jz_stage_v.cu", "jz_stage_common.cuh", "jz_fastmath.cuh", "jz_common.cuh", "jz_api.cu"),
                  1: ("jz_stage.cu", "jz_stage_common.cuh", "jz_fastmath.cuh", "jz_common.cuh", "jz_api.cu"),
-                 0: ("jz_stage.cu", "jz_stage_common.cuh", "jz_fastmath.cuh", "jz_common.cuh", "jz_api.cu")}
+                 0: ("jz_stage_d.cu", "jz_stage_common.cuh", "jz_fastmath.cuh", "jz_common.cuh", "jz_api.cu")}
 STAGE_KERNELS = {2: "k_stage_v (fused RK stage, vector node records)",
                  1: "k_stage<float,double,32,16> (fused RK stage)",
-                 0: "k_stage<double,double,16,16> (fused RK stage)"}
+                 0: "k_stage_d (fused RK stage, FP64)"}
 
 
 def stage_source_sha(prec: int) -> str:

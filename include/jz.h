@@ -429,7 +429,7 @@ int jz_set_tiling(jz_grid* g, int kc);
  * float4 + float vectors in shared memory (two block barriers per plane);
  * 0 is the scalar kernel (one shared-memory value per load, four barriers
  * per plane).  Both evaluate the same formulas; results agree to FP32
- * rounding.  Measured on the 256x192x192 mapped jet: 0.41 ms (2) and 0.55 ms
+ * rounding.  Measured on the 256x192x192 mapped jet: 0.30 ms (2) and 0.55 ms
  * (0) per stage.  Grids of the other precision modes run one kernel only (the
  * scalar one for JZ_P64 and JZ_P32_M64, the vector-record one for
  * JZ_P32_S64): variant 0 is accepted there without effect; JZ_EINVAL for

@@ -45,12 +45,13 @@
 // its own, the kernel moved 7.8 shared-memory wavefronts per point through a
 // pipe 67% busy and stalled 0.9 cycles per instruction on instruction fetch
 // (103 KB of code for the three roles).  The column in tensor memory took the
-// wavefronts to 6.1, and the single loop body the code to 42 KB, the fetch
-// stalls to 0.2 and the issue rate from 53% to 65%: 0.360 to 0.301 ms per
-// stage on 256x192x192 (c1).  Tensor memory alone, with the old code size,
-// gained 1%: the fetch stalls rose by what the memory stalls fell.  Now issue
-// slots (65%) and the shared-memory pipe (64%) bind together, with the
-// barriers between.
+// wavefronts to 6.0, and the single loop body the code to 42 KB, the fetch
+// stalls to 0.2 and the issue rate from 53% to 66%: 1.98 to 1.72 ms per step
+// on 256x192x192.  Tensor memory alone, with the old code size, gained 1%: the
+// fetch stalls rose by what the memory stalls fell.  Block barriers without a
+// reduction and the set-up before the previous kernel's end took the step to
+// 1.69 ms (a stage 0.361 to 0.302 ms).  Now issue slots (66%) and the shared-memory
+// pipe (64%) bind together, with the barriers between.
 #include <cmath>
 #include <cstdint>
 
@@ -574,6 +575,7 @@ __device__ __forceinline__ bool item_v(const StageCtx<float, float>& X, const KC
   // generic-proxy writes to the buffers the prologue stages into, then the barrier
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
+  // up to here parameters and shared memory only
   if (first) wait_for_previous();
 
   // thread 0's record of its copies: bit b of pend = barrier b has had one,
@@ -954,7 +956,9 @@ template <int MD, bool S64>
 __global__ void __launch_bounds__(vr::NT, vr::MINB)
     k_stage_v(const __grid_constant__ StageCtx<float, float> X, const StageSel st) {
   extern __shared__ __align__(128) unsigned char smem[];
-  if (threadIdx.x == 0) {  // with the barriers' set-up, before the previous kernel's results are needed
+  // with the barriers' set-up, before the previous kernel's results are needed:
+  // 69x47x46 90.3 to 88.2 us per step, 256x192x192 1.697 to 1.686 ms
+  if (threadIdx.x == 0) {
     prefetch_map(&X.tmQ[st.qin]);
     prefetch_map(&X.tmMv);
     prefetch_map(&X.tmQ0u);
