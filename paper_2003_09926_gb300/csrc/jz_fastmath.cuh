@@ -10,7 +10,8 @@ namespace stg {
 
 // Elementary functions.  FP32 arithmetic uses the hardware approximations
 // (sqrt.approx, rcp.approx, ex2/lg2.approx: a few ulp, far below the FP32
-// error of the scheme itself); FP64 arithmetic keeps IEEE operations.
+// error of the scheme itself); Fn<double> is the library's (boundary pass,
+// Vreman's model), the FP64 kernels' own functions follow it.
 template <typename R> struct Fn;
 template <> struct Fn<float> {
   static __device__ __forceinline__ float sqrt_(float x) {
@@ -55,30 +56,61 @@ template <> struct Fn<double> {
   }
 };
 
-// FP64 reciprocal and square root from the hardware's approximations and one
-// third-order step, written from their series; 3 and 5 FP64 instructions, a
-// half to a quarter of the correctly rounded forms', on a pipe that passes two
-// lanes per cycle and SM.  Error below 1.5 units in the last place.
+// FP64 reciprocal, square root and J^(-2/3) of the FP64 stage kernel and
+// time-step reduction, whose FP64 pipe passes two lanes per cycle and SM: from
+// the hardware's approximations (relative error e of 2^-19.9 for rcp and
+// 2^-19.0 for rsqrt, the largest seen over 2^26 mantissas) and their Taylor
+// series to e^3, 4, 7 and 7 FP64 instructions.  What the series leave out is below
+// 2^-75, so that reciprocal and square root err by the last rounding alone
+// (0.5 units in the last place) and J^(-2/3) by it and two thirds of the one in
+// y^3, less than the library's cbrt, product and division (1.01 against 3.2
+// units).  Step of a 128x96x96 grid: 6.26 ms, 6.63 with the library's division,
+// square root and cbrt, 5.98 with the series to e^2, which err by 0.504, 0.75
+// and 2.3 units.
 
-// 1/b: with e = 1 - b y of an approximation y, 1/b = y (1 + e + e^2 + ...);
-// |e| < 2^-20, so what is left out is below 2^-60.
-__device__ __forceinline__ double rcp3(double b) {
+// 1/b: with e = 1 - b y, 1/b = y (1 + e + e^2 + e^3 + ...)
+__device__ __forceinline__ double rcp_d(double b) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
   const double e = fma(-b, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  return fma(y, fma(fma(e, e, e), e, e), y);
 }
 
-// sqrt(x): with e = 1 - x y^2 of an approximation y to x^(-1/2) and t = x y,
-// sqrt(x) = t (1 + e/2 + 3 e^2/8 + ...); |e| < 2^-20.  Zero (tested on the bits,
-// where y is infinite) gives zero.
-__device__ __forceinline__ double sqrt3(double x) {
+// sqrt(x): y of an approximation to x^(-1/2), t + l = x y exactly; with
+// e = 1 - t y, sqrt(x) = t + (t e + l) (1/2 + 3 e/8 + 5 e^2/16 + ...).  Zero
+// (tested on the bits, where y is infinite) gives zero.
+__device__ __forceinline__ double sqrt_d(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double t = __dmul_rn(x, y);
+  const double l = fma(x, y, -t);
   const double e = fma(-t, y, 1.0);
-  const double r = fma(__dmul_rn(t, e), fma(0.375, e, 0.5), t);
+  const double r = fma(fma(t, e, l), fma(fma(0.3125, e, 0.375), e, 0.5), t);
   return (uint32_t)(__double2hiint(x) & 0x7fffffff) < 0x00100000u ? 0.0 : r;
+}
+
+// J^(-2/3) (of |J|): J = m 2^(3q), 1 <= m < 16; y of an FP32 approximation to
+// m^(-1/3) (y^2 is exact in FP64), then with e = 1 - m y^3,
+// m^(-2/3) = y^2 (1 + 2 e/3 + 5 e^2/9 + 40 e^3/81 + ...).  The exponents are
+// integer arithmetic.
+__device__ __forceinline__ double jm23_d(double J) {
+  const int hi = __double2hiint(J) & 0x7fffffff, lo = __double2loint(J);
+  const int ex = (hi >> 20) - 1023;
+  const int q = (ex * 21846) >> 16;  // floor(ex / 3), or one less
+  const double m = __hiloint2double(hi - (q * 3 << 20), lo);
+  float y, l;
+  asm("lg2.approx.ftz.f32 %0, %1;"
+      : "=f"(l)
+      : "f"(__uint_as_float((((uint32_t)hi & 0xfffffu) << 3 | (uint32_t)lo >> 29) | (uint32_t)(ex - 3 * q + 127) << 23)));
+  l *= -1.0f / 3.0f;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(l));
+  const uint32_t b = __float_as_uint(y);  // a normal number: widened by its bits
+  const double y1 = __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+  const double y2 = __dmul_rn(y1, y1);
+  const double e = fma(-m, __dmul_rn(y2, y1), 1.0);
+  const double c = fma(fma(40.0 / 81.0, e, 5.0 / 9.0), e, 2.0 / 3.0);
+  const double r = fma(__dmul_rn(y2, e), c, y2);
+  return __hiloint2double(__double2hiint(r) - (q * 2 << 20), __double2loint(r));
 }
 
 }  // namespace stg

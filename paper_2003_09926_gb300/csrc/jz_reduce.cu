@@ -33,14 +33,14 @@ int red_grid(int per_sm) {
 // reciprocal and square root of the reduction: IEEE in FP32 (bound by memory),
 // the short forms in FP64 (bound by the FP64 pipe)
 __device__ __forceinline__ float rd_rcp(float x) { return 1.f / x; }
-__device__ __forceinline__ double rd_rcp(double x) { return stg::rcp3(x); }
+__device__ __forceinline__ double rd_rcp(double x) { return stg::rcp_d(x); }
 __device__ __forceinline__ float rd_sqrt(float x) { return sqrt(x); }
-__device__ __forceinline__ double rd_sqrt(double x) { return stg::sqrt3(x); }
+__device__ __forceinline__ double rd_sqrt(double x) { return stg::sqrt_d(x); }
 __device__ __forceinline__ float sutherland(float mu_inf, float s1, float temp, float root) {
   return mu_inf * temp * root * (1.f + s1) / (temp + s1);
 }
 __device__ __forceinline__ double sutherland(double mu_inf, double s1, double temp, double root) {
-  return mu_inf * temp * root * (1.0 + s1) * stg::rcp3(temp + s1);
+  return mu_inf * temp * root * (1.0 + s1) * stg::rcp_d(temp + s1);
 }
 
 __device__ __forceinline__ double warp_max(double v) {

@@ -23,9 +23,8 @@
 //  - gradients left without their factor J/2, which multiplies the two
 //    viscosities instead of twelve gradients;
 //  - reciprocals, square roots and J^(-2/3) from the hardware's 20-bit (FP64)
-//    or FP32 approximations and one third-order step each (3, 5 and 7
-//    instructions; the library's correctly rounded forms take two to four
-//    times as many);
+//    or FP32 approximations and one fourth-order step each (4, 7 and 7
+//    instructions: 6% of a step less than the library's forms, as precise);
 //  - the planes below and above a chunk and its halo nodes there, which only
 //    build up the march, form their k quantities only.
 // All FP64 arithmetic is written as explicit rounded operations, so that a
@@ -45,29 +44,6 @@ namespace {
 __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
-
-// J^(-2/3) (of |J|): J = m 2^(3q), 1 <= m < 16; y of an FP32 approximation to
-// m^(-1/3), then with e = 1 - m y^3, m^(-1/3) = y (1 + e/3 + 2 e^2/9 + ...);
-// |e| < 2^-18, so what is left out is below 2^-56.  The exponents are integer
-// arithmetic.
-__device__ __forceinline__ double jm23_3(double J) {
-  const int hi = __double2hiint(J) & 0x7fffffff, lo = __double2loint(J);
-  const int ex = (hi >> 20) - 1023;
-  const int q = (ex * 21846) >> 16;  // floor(ex / 3), or one less
-  const double m = __hiloint2double(hi - (q * 3 << 20), lo);
-  float y, l;
-  asm("lg2.approx.ftz.f32 %0, %1;"
-      : "=f"(l)
-      : "f"(__uint_as_float((((uint32_t)hi & 0xfffffu) << 3 | (uint32_t)lo >> 29) | (uint32_t)(ex - 3 * q + 127) << 23)));
-  l *= -1.0f / 3.0f;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(l));
-  const uint32_t b = __float_as_uint(y);  // a normal number: widened by its bits
-  const double y0 = __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
-  const double e = fma(-m, mul(mul(y0, y0), y0), 1.0);
-  const double y1 = fma(mul(y0, e), fma(2.0 / 9.0, e, 1.0 / 3.0), y0);
-  const double r = mul(y1, y1);
-  return __hiloint2double(__double2hiint(r) - (q * 2 << 20), __double2loint(r));
-}
 
 // the larger of two numbers, compared by their bits (an order-preserving map
 // to signed integers)
@@ -198,7 +174,7 @@ struct Node {
     for (int f = 0; f < 9; ++f) S[f] = met[f * MPL + mo];
     J = met[9 * MPL + mo];
     const double u = pc[0], v = pc[1], w = pc[2], T = pc[3];
-    const double cson = sqrt3(T);
+    const double cson = sqrt_d(T);
 #pragma unroll
     for (int m = 0; m < 3; ++m)
 #pragma unroll
@@ -215,7 +191,7 @@ struct Node {
         for (int m = 0; m < 3; ++m) g[q][m] = fma(S[6 + m], d2, fma(S[3 + m], d1, mul(S[m], d0)));
       }
       const double hJ = mul(0.5, J);
-      const double mu = mul(mul(k.muc, mul(T, cson)), rcp3(add(T, c.s1)));  // Sutherland
+      const double mu = mul(mul(k.muc, mul(T, cson)), rcp_d(add(T, c.s1)));  // Sutherland
       const double s01 = add(g[0][1], g[1][0]), s02 = add(g[0][2], g[2][0]), s12 = add(g[1][2], g[2][1]);
       double mu_t = 0.0;
       if (ModelFlags<MD>::sgs(c)) {
@@ -230,7 +206,7 @@ struct Node {
         } else {  // Smagorinsky: (C_s Delta)^2 sqrt(2 S_ij S_ij), Delta^2 = J^(-2/3)
           const double dd = fma(g[2][2], g[2][2], fma(g[1][1], g[1][1], mul(g[0][0], g[0][0])));
           const double ss = fma(2.0, dd, fma(s12, s12, fma(s02, s02, mul(s01, s01))));
-          nu_t = mul(mul(c.cs2, mul(sqrt3(ss), hJ)), jm23_3(J));
+          nu_t = mul(mul(c.cs2, mul(sqrt_d(ss), hJ)), jm23_d(J));
         }
         mu_t = mul(rho, nu_t);
       }
@@ -247,8 +223,8 @@ struct Node {
     for (int d = 0; d < 3; ++d) {
       U[d] = fma(S[3 * d + 2], w, fma(S[3 * d + 1], v, mul(S[3 * d], u)));
       const double s2 = fma(S[3 * d + 2], S[3 * d + 2], fma(S[3 * d + 1], S[3 * d + 1], mul(S[3 * d], S[3 * d])));
-      lam[d] = fma(cson, sqrt3(s2), fabs(U[d]));
-      sq[d] = ModelFlags<MD>::sig_half(c) ? sqrt3(lam[d]) : 0.0;
+      lam[d] = fma(cson, sqrt_d(s2), fabs(U[d]));
+      sq[d] = ModelFlags<MD>::sig_half(c) ? sqrt_d(lam[d]) : 0.0;
     }
   }
   // G^d = E^d - F^d, lambda~^d and nu^d of one direction with face vector
@@ -269,7 +245,7 @@ struct Node {
       G[5] = fma(sl, add(sa, sb), l);
     else
       G[5] = l > 0.0 ? mul(l, add(add(1.0, pow(la / l, c.sigma)), pow(lb / l, c.sigma))) : 0.0;
-    G[6] = mul(fabs(add(fma(-2.0, p, pp), pm)), rcp3(add(fma(2.0, p, pp), pm)));
+    G[6] = mul(fabs(add(fma(-2.0, p, pp), pm)), rcp_d(add(fma(2.0, p, pp), pm)));
   }
 };
 
@@ -402,7 +378,7 @@ __device__ __forceinline__ bool item_d(const StageCtx<double, double>& X, const 
       if (on) {
 #pragma unroll
         for (int v = 0; v < 5; ++v) r[5 + v] = src[v * PL + e];
-        const double ri = rcp3(r[5]);
+        const double ri = rcp_d(r[5]);
 #pragma unroll
         for (int m = 0; m < 3; ++m) r[m] = mul(r[6 + m], ri);
         const double k2 = fma(r[2], r[8], fma(r[1], r[7], mul(r[0], r[6])));  // rho |u|^2
