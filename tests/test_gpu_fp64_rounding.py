@@ -1,6 +1,6 @@
-"""The FP64 elementary functions that the FP64 kernels evaluate from the
-hardware's approximations, against extended precision over mantissas and
-exponents."""
+"""Rounding errors of the FP64 kernels' building blocks, against extended
+precision: the elementary functions that they evaluate from the hardware's
+approximations, over mantissas and exponents, and the face flux."""
 import ctypes as C
 import os
 import subprocess
@@ -13,24 +13,35 @@ pytestmark = pytest.mark.gpu
 RCP, SQRT, JM23, JM23_LIBRARY = range(4)
 
 
-@pytest.fixture(scope="module")
-def evaluate(tmp_path_factory):
+P = C.POINTER(C.c_double)
+
+
+def _dp(a):
+    return a.ctypes.data_as(P)
+
+
+def _probe(tmp_path_factory, name):
+    """tests/probes/<name>.cu, which includes the kernels' source, as a library."""
     import torch
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2003_09926_gb300 import build
-    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "probes", "fastmath_probe.cu")
-    lib = str(tmp_path_factory.mktemp("probe") / "fastmath_probe.so")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "probes", name + ".cu")
+    lib = str(tmp_path_factory.mktemp("probe") / (name + ".so"))
     subprocess.run([build.nvcc(), *build.ARCH, "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-shared", "-o", lib, src],
                    check=True)
-    fn = C.CDLL(lib).fastmath_eval
-    P = C.POINTER(C.c_double)
+    return C.CDLL(lib)
+
+
+@pytest.fixture(scope="module")
+def evaluate(tmp_path_factory):
+    fn = _probe(tmp_path_factory, "fastmath_probe").fastmath_eval
     fn.argtypes = [C.c_int, C.c_int, P, P]
 
     def run(which, x):
         x = np.ascontiguousarray(x, dtype=np.float64)
         y = np.empty_like(x)
-        assert fn(which, x.size, x.ctypes.data_as(P), y.ctypes.data_as(P)) == 0
+        assert fn(which, x.size, _dp(x), _dp(y)) == 0
         return y
 
     return run
@@ -77,3 +88,31 @@ def test_power_minus_two_thirds(evaluate):
     err, library = _ulps(evaluate(JM23, x), exact), _ulps(evaluate(JM23_LIBRARY, x), exact)
     assert err.max() <= 0.5 + 2.0 / 3.0 + 2.0 ** -10
     assert np.sqrt((err ** 2).mean()) <= np.sqrt((library ** 2).mean())
+
+
+def test_face_flux_rounds_once_at_the_size_of_the_sum(tmp_path_factory):
+    """2h = Ga + Gb - l2 d1 + l4 d3 with Ga, Gb in [1, 1.9] and a dissipation
+    below 2^-10 of them.  Of the three roundings one is of the sum (in [2, 4):
+    2^-52 at most) and two of Ga and Gb with their share of the dissipation
+    (in [1, 2): 2^-53 each): 2^-51, and below 2^-60 from the dissipation's own
+    roundings.  Adding the dissipation to the sum would round three times at
+    its size, up to 1.5 2^-51."""
+    fn = _probe(tmp_path_factory, "face_probe").face_eval
+    fn.argtypes = [C.c_int, C.c_double, C.c_double, P, P]
+    n, k2, k4 = 200_000, 0.25, 2.0 ** -8
+    rng = np.random.default_rng(3)
+    x = np.empty((n, 34))
+    x[:, :14] = 1.0 + 0.9 * rng.random((n, 14))
+    x[:, [5, 12]] = 0.5 * rng.random((n, 2))  # radii
+    x[:, [6, 13]] = 0.01 * rng.random((n, 2))  # sensors
+    x[:, 14:] = 1.0 + 2.0 ** -6 * rng.random((n, 20))
+    y = np.empty((n, 5))
+    assert fn(n, k2, k4, _dp(x), _dp(y)) == 0
+    L = x.astype(np.longdouble)
+    Ga, Gb = L[:, 0:5], L[:, 7:12]
+    qm, qa, qb, qp = (L[:, 14 + 5 * m:19 + 5 * m] for m in range(4))
+    lam = (L[:, 5] + L[:, 12])[:, None]
+    e2 = k2 * np.maximum(L[:, 6], L[:, 13])[:, None]
+    e4 = np.maximum(0.0, k4 - e2)
+    exact = Ga + Gb - lam * (e2 * (qb - qa) - e4 * (qp - 3 * qb + 3 * qa - qm))
+    assert np.abs(y - exact).max() <= 2.0 ** -51 * (1.0 + 2.0 ** -8)
