@@ -90,15 +90,20 @@ def test_power_minus_two_thirds(evaluate):
     assert np.sqrt((err ** 2).mean()) <= np.sqrt((library ** 2).mean())
 
 
-def test_face_flux_rounds_once_at_the_size_of_the_sum(tmp_path_factory):
+@pytest.fixture(scope="module")
+def face(tmp_path_factory):
+    fn = _probe(tmp_path_factory, "face_probe").face_eval
+    fn.argtypes = [C.c_int, C.c_double, C.c_double, P, P]
+    return fn
+
+
+def test_face_flux_rounds_once_at_the_size_of_the_sum(face):
     """2h = Ga + Gb - l2 d1 + l4 d3 with Ga, Gb in [1, 1.9] and a dissipation
     below 2^-10 of them.  Of the three roundings one is of the sum (in [2, 4):
     2^-52 at most) and two of Ga and Gb with their share of the dissipation
     (in [1, 2): 2^-53 each): 2^-51, and below 2^-60 from the dissipation's own
     roundings.  Adding the dissipation to the sum would round three times at
     its size, up to 1.5 2^-51."""
-    fn = _probe(tmp_path_factory, "face_probe").face_eval
-    fn.argtypes = [C.c_int, C.c_double, C.c_double, P, P]
     n, k2, k4 = 200_000, 0.25, 2.0 ** -8
     rng = np.random.default_rng(3)
     x = np.empty((n, 34))
@@ -107,7 +112,7 @@ def test_face_flux_rounds_once_at_the_size_of_the_sum(tmp_path_factory):
     x[:, [6, 13]] = 0.01 * rng.random((n, 2))  # sensors
     x[:, 14:] = 1.0 + 2.0 ** -6 * rng.random((n, 20))
     y = np.empty((n, 5))
-    assert fn(n, k2, k4, _dp(x), _dp(y)) == 0
+    assert face(n, k2, k4, _dp(x), _dp(y)) == 0
     L = x.astype(np.longdouble)
     Ga, Gb = L[:, 0:5], L[:, 7:12]
     qm, qa, qb, qp = (L[:, 14 + 5 * m:19 + 5 * m] for m in range(4))
@@ -116,3 +121,19 @@ def test_face_flux_rounds_once_at_the_size_of_the_sum(tmp_path_factory):
     e4 = np.maximum(0.0, k4 - e2)
     exact = Ga + Gb - lam * (e2 * (qb - qa) - e4 * (qp - 3 * qb + 3 * qa - qm))
     assert np.abs(y - exact).max() <= 2.0 ** -51 * (1.0 + 2.0 ** -8)
+
+
+def test_zero_infinity_and_nan(evaluate):
+    """As in IEEE arithmetic, with subnormal numbers taken as zero."""
+    inf, nan, tiny, big = np.inf, np.nan, 2.0 ** -1030, np.finfo(np.float64).max
+    x = np.array([0.0, -0.0, inf, -inf, nan, -nan, tiny, -tiny])
+    np.testing.assert_array_equal(evaluate(RCP, x), [inf, -inf, 0.0, -0.0, nan, nan, inf, -inf])
+    np.testing.assert_array_equal(np.signbit(evaluate(RCP, x[2:4])), [False, True])
+    x = np.array([0.0, -0.0, inf, -inf, nan, -nan, tiny, -1.0, -big])
+    np.testing.assert_array_equal(evaluate(SQRT, x), [0.0, 0.0, inf, nan, nan, nan, 0.0, nan, nan])
+    x = np.array([0.0, inf, nan, -nan, tiny])
+    np.testing.assert_array_equal(evaluate(JM23, x), [inf, 0.0, nan, nan, inf])
+    # the ends of the normal numbers
+    x = np.array([2.0 ** -1022, 2.0 ** 1021, big, 2.0 ** 1023])
+    np.testing.assert_allclose(evaluate(RCP, x), 1.0 / x, rtol=2.0 ** -52, atol=2.0 ** -1022)
+    np.testing.assert_array_equal(evaluate(SQRT, x), np.sqrt(x))
