@@ -46,11 +46,12 @@ __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, 
 __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
 
 // the larger of two numbers, compared by their bits (an order-preserving map
-// to signed integers)
-__device__ __forceinline__ double max_bits(double a, double b) {
-  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
-  return (x ^ ((x >> 63) & 0x7fffffffffffffffLL)) > (y ^ ((y >> 63) & 0x7fffffffffffffffLL)) ? a : b;
+// to signed integers); a NaN of either sign is larger than any number
+__device__ __forceinline__ long long order_bits(double a) {
+  const long long x = __double_as_longlong(a);
+  return (__double2hiint(a) & 0x7fffffff) > 0x7ff00000 ? 0x7fffffffffffffffLL : x ^ ((x >> 63) & 0x7fffffffffffffffLL);
 }
+__device__ __forceinline__ double max_bits(double a, double b) { return order_bits(a) > order_bits(b) ? a : b; }
 
 template <int TI_, int TJ_>
 struct Cfg {

@@ -137,3 +137,20 @@ def test_zero_infinity_and_nan(evaluate):
     x = np.array([2.0 ** -1022, 2.0 ** 1021, big, 2.0 ** 1023])
     np.testing.assert_allclose(evaluate(RCP, x), 1.0 / x, rtol=2.0 ** -52, atol=2.0 ** -1022)
     np.testing.assert_array_equal(evaluate(SQRT, x), np.sqrt(x))
+
+
+def test_a_nan_sensor_reaches_the_face_flux(face):
+    """Whichever side of a face has it, and whatever its sign: the state then
+    shows it instead of going on with the other side's dissipation."""
+    n = 4
+    x = np.ones((n, 34))
+    x[:, [6, 13]] = 0.01
+    x[0, 6], x[1, 6] = np.nan, -np.nan
+    x[2, 13], x[3, 13] = np.nan, -np.nan
+    y = np.zeros((n, 5))
+    assert face(n, 0.25, 2.0 ** -8, _dp(x), _dp(y)) == 0
+    assert np.isnan(y).all()
+    x[:, [6, 13]] = [[0.01, np.inf], [np.inf, 0.01], [-0.5, 0.01], [0.01, -0.5]]
+    x[:, 24] = 1.5  # a density jump at the face
+    assert face(n, 0.25, 2.0 ** -8, _dp(x), _dp(y)) == 0
+    assert not np.isfinite(y[:2, 0]).any() and np.isfinite(y[2:]).all()
