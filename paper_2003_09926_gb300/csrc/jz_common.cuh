@@ -182,7 +182,9 @@ template <> struct RunSum<float> {
 // stream has flushed its results, once its blocks have all exited or called
 // let_next_start(); every such kernel calls wait_for_previous() before it
 // touches global memory (results of the kernels before are then visible, since
-// the previous kernel waited too).  It takes 0.4 us per launch off the chain
+// the previous kernel waited too).  Arrays that a kernel of a step writes are
+// read through plain pointers there: const __restrict__ ones allow non-coherent
+// loads, which the compiler may also move above the wait.  It takes 0.4 us per launch off the chain
 // of eleven: 69x47x46, 98 to 94 us per step.  let_next_start() at the start of
 // the stage kernel measured slower (its waiting successors, 1.72 to 1.75 ms on
 // 256x192x192), so only the short kernels call it: the boundary pass while it

@@ -644,7 +644,7 @@ constexpr int fill_threads() { return sizeof(ST) == 8 ? 64 : (CYL ? 32 * AX_WARP
 template <typename ST, typename MT, bool FAST, bool CYL>
 __global__ void __launch_bounds__(fill_threads<ST, CYL>(), CYL ? 3 : 1)
     k_bc_fill(const __grid_constant__ Layout L, const __grid_constant__ Slabs sl, const __grid_constant__ FillBlocks fb,
-              const double* __restrict__ inflow, const double* __restrict__ axis, const __grid_constant__ FlowC F,
+              const double* __restrict__ inflow, const double* axis, const __grid_constant__ FlowC F,
               ST* __restrict__ Q, const MT* __restrict__ M) {
   constexpr bool AXIS_IN = CYL && sizeof(ST) == 4;
   if (fb.one_wave) let_next_start();

@@ -161,7 +161,7 @@ struct DiagAcc {
 // record after the RED_BLOCKS rate partials) and the last block publishes
 // them, as k_diag does.
 template <typename ST, typename MT, bool DIAG = false>
-__device__ __forceinline__ void timestep_body(const Layout& L, const FlowC& F, const ST* __restrict__ Q,
+__device__ __forceinline__ void timestep_body(const Layout& L, const FlowC& F, const ST* Q,
                                               const MT* __restrict__ M, Scalars* sc, double* partial, double cfl,
                                               bool finalize = true) {
   const ST g = flow_const<ST>(F.gamma, F.gamma_f), gm1 = flow_const<ST>(F.gm1, F.gm1_f);
@@ -292,7 +292,7 @@ __device__ __forceinline__ void timestep_body(const Layout& L, const FlowC& F, c
 }
 
 template <typename ST, typename MT, bool DIAG = false>
-__global__ void __launch_bounds__(RED_THREADS) k_timestep(Layout L, FlowC F, const ST* __restrict__ Q,
+__global__ void __launch_bounds__(RED_THREADS) k_timestep(Layout L, FlowC F, const ST* Q,
                                                           const MT* __restrict__ M, Scalars* sc, double* partial,
                                                           double cfl, bool finalize) {
   wait_for_previous();
