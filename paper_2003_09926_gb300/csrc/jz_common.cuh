@@ -184,12 +184,12 @@ template <> struct RunSum<float> {
 // touches global memory (results of the kernels before are then visible, since
 // the previous kernel waited too).  Arrays that a kernel of a step writes are
 // read through plain pointers there: const __restrict__ ones allow non-coherent
-// loads, which the compiler may also move above the wait.  It takes 0.4 us per launch off the chain
-// of eleven: 69x47x46, 98 to 94 us per step.  let_next_start() at the start of
-// the stage kernel measured slower (its waiting successors, 1.72 to 1.75 ms on
-// 256x192x192), so only the short kernels call it: the boundary pass while it
-// is one wave of blocks (94 to 92 us; with several waves 0.2% slower) and the
-// time-step reduction after its loop.
+// loads, which the compiler may also move above the wait.  It takes 0.4 us per
+// launch off the chain of eleven: 69x47x46, 98 to 94 us per step.
+// let_next_start() at the start of the stage kernel measured slower (its waiting
+// successors, 1.72 to 1.75 ms on 256x192x192), so only the short kernels call it:
+// the boundary pass up to 8 blocks per SM (94 to 92 us; with more 0.2% slower) and
+// the time-step reduction after its loop.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... KA, typename... A>
