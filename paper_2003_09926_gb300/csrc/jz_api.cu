@@ -918,7 +918,7 @@ void batch_chunks(jz_grid* const* grids, int n, StageTiling t, std::vector<int>&
     const Layout& L = grids[k]->dev.L;
     g[k].tiles = (long long)((L.hi[0] + t.ti) / t.ti) * ((L.hi[1] + t.tj) / t.tj);
     g[k].nz = L.hi[2] - L.lo[2] + 1;
-    g[k].fixed = grids[k]->dev.kc_set ? grids[k]->dev.kc : 0;
+    g[k].fixed = grids[k]->dev.kc_set ? std::min(grids[k]->dev.kc, g[k].nz) : 0;
     g[k].k = k;
     g[k].work = g[k].tiles * g[k].nz;
     longest = std::max(longest, g[k].nz);

@@ -37,6 +37,7 @@
 //    Q^(0) held in registers;
 //  - every configuration is compiled for the Smagorinsky flow model of the
 //    workloads with constant flags and once with the flags read at run time.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -596,7 +597,7 @@ void fill_ctx(StageCtx<R, MT>& X, const GridDev& g) {
   X.err = &g.sc->err;
   X.F = g.F;
   X.k = make_kconst<R>(g.F);
-  X.kc = g.kc;
+  X.kc = std::min(g.kc, g.L.hi[2] - g.L.lo[2] + 1);  // a longer chunk is the whole column
 }
 
 template <typename R, typename MT, int TI, int TJ>
@@ -606,7 +607,7 @@ cudaError_t launch_one(const GridDev& g, int stage, int qsel, int qout, cudaStre
   fill_ctx(X, g);
   const StageSel st{kRkAlpha[stage], qsel, qout, g.stall_test};
   const int nz = g.L.hi[2] - g.L.lo[2] + 1;
-  dim3 grid((g.L.hi[0] + TI) / TI, (g.L.hi[1] + TJ) / TJ, (nz + g.kc - 1) / g.kc);
+  dim3 grid((g.L.hi[0] + TI) / TI, (g.L.hi[1] + TJ) / TJ, (nz + X.kc - 1) / X.kc);
   if (flow_model(X.k) == kModelSmagorinsky)
     k_stage<R, MT, TI, TJ, kModelSmagorinsky><<<grid, Cf::NT, Cf::BYTES, s>>>(X, st);
   else
