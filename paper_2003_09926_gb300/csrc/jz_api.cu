@@ -903,11 +903,12 @@ StageTiling batch_tiling(const GridDev& d) { return d.prec == JZ_P64 ? StageTili
 // chunks short enough to fill the device by itself; in a batch the other
 // grids do that, and every chunk costs about three planes more than it
 // updates.  So each grid whose length was not set (jz_set_tiling) is cut into
-// the same number of chunks of at most `len` planes, len the one of the
-// largest grid's 1/1, 1/2, 1/3, ... that gives the shortest makespan of the
-// queue (simulated: resident CTAs taking items in queue order, an item's cost
-// its planes plus three).  Finer cuts stop paying once the queue holds many
-// items per CTA.  64 grids of up to 160x128x128 (FP32): 11.09 ms per step with
+// equal chunks of at most `len` planes, len the one of the largest column's 1/1,
+// 1/2, 1/3, ... that gives the shortest makespan of the queue (simulated:
+// resident CTAs taking items in queue order, an item's cost its planes plus
+// three).  Finer cuts stop paying once the queue holds many items per CTA.  The
+// search takes 1 to 12 us of host time, twice for a batch made (its bytes, then
+// the batch).  64 grids of up to 160x128x128 (FP32): 11.09 ms per step with
 // the single-grid lengths, 10.13 ms with these (whole columns);
 // four grids 0.46 and 0.39 ms (about a dozen planes).
 void batch_chunks(jz_grid* const* grids, int n, StageTiling t, std::vector<int>& kc) {
@@ -933,24 +934,33 @@ void batch_chunks(jz_grid* const* grids, int n, StageTiling t, std::vector<int>&
     const int c = (x.nz + len - 1) / len;
     return (x.nz + c - 1) / c;
   };
-  int best_len = longest;
-  long long best = -1;
-  for (int cut = 1; cut <= 32; ++cut) {
+  int best_len = longest, last = 0;
+  long long best = -1, planes = 0;
+  bool chosen = false;  // some length is to be chosen
+  for (const G& x : g) {
+    planes += x.work;
+    chosen = chosen || !x.fixed;
+  }
+  std::vector<long long> ctas;  // by finishing time
+  for (int cut = 1; cut <= 32 && chosen; ++cut) {
     const int len = (longest + cut - 1) / cut;
     if (len < 2 && cut > 1) break;
-    long long items = 0;
-    for (const G& x : g) items += x.tiles * ((x.nz + chunk(x, len) - 1) / chunk(x, len));
-    if (cut > 1 && items > 24 * slots) break;
-    // the CTAs counted by finishing time (whole planes): an item goes to one
-    // that is free first, and a chunk of a grid's tiles to many at once (item by
-    // item on a heap of CTAs this took 0.1 to 2.6 ms of every batch made)
-    long long total = 0, longest_item = 0;
+    if (len == last) continue;
+    last = len;
+    long long items = 0, longest_item = 0;
     for (const G& x : g) {
       const int l = chunk(x, len);
-      total += x.tiles * (x.nz + 3LL * ((x.nz + l - 1) / l));
+      items += x.tiles * ((x.nz + l - 1) / l);
       longest_item = std::max(longest_item, std::min(l, x.nz) + 3LL);
     }
-    std::vector<long long> ctas(total / slots + longest_item + 1, 0);
+    if (cut > 1 && items > 24 * slots) break;
+    // no order takes less than the total over the CTAs, and a finer cut's total
+    // is no smaller: once it is the best span's, the search ends
+    const long long total = planes + 3 * items;
+    if (best >= 0 && (total + slots - 1) / slots >= best) break;
+    // the CTAs counted by finishing time (whole planes): an item goes to one
+    // that is free first, and a chunk of a grid's tiles to many at once
+    ctas.assign(total / slots + longest_item + 1, 0);
     ctas[0] = slots;
     long long now = 0, span = 0;  // no CTA is free before now
     for (const G& x : g) {
