@@ -9,9 +9,12 @@ across SMs, long chunks amortise each chunk's prologue (four staged planes
 and two node passes); a narrow tile wastes fewer padded columns on a grid
 narrow in i, a small one on a small grid.  Both are chosen here by timing
 candidates on scratch grids of the same shape (the caller's state is
-untouched) with CUDA events; other precision modes have a fixed (i, j) tile
-and only kc is tuned.  Results are cached per (precision, shape) for single
-grids and per batch signature for batches, where one shape serves every grid.
+untouched) with CUDA events; in other precision modes the library sets the
+(i, j) tile and only kc is tuned.  The length that the library itself chooses
+is always one of the candidates: a grid's default, and for a batch the lengths
+chosen for the whole batch (CHOSEN).  Results are cached per (precision, shape)
+for single grids and per batch signature for batches, where one shape serves
+every grid.
 """
 from __future__ import annotations
 
@@ -19,6 +22,7 @@ from . import jz
 
 SHAPES = ((32, 16), (16, 32), (16, 16))
 P32 = 2  # the precision mode whose default kernel has selectable tile shapes
+CHOSEN = -1  # k-chunk length of a choice: the ones the library chooses
 
 _cache: dict = {}
 
@@ -53,7 +57,7 @@ def _shapes(desc: dict):
 
 def apply(grid: jz.Grid, choice: dict) -> None:
     """Set a tuned choice {"shape": (ti, tj) or None, "kc": planes (0 = whole
-    k range)} on a grid."""
+    k range, CHOSEN = left to the library)} on a grid."""
     if choice.get("shape") is not None:
         jz.jz_set_tile_shape(grid.h, *choice["shape"])
     apply_kc(grid, choice["kc"])
@@ -73,7 +77,8 @@ def tune_grid(desc: dict, flow: dict, cfl: float = 0.5, reps: int = 3, device: i
     for shape in _shapes(desc):
         if shape is not None:
             jz.jz_set_tile_shape(g.h, *shape)
-        for kc in candidates_for(_nz(desc)):
+        default = jz.jz_get_tiling(g.h)[2]
+        for kc in [default] + [c for c in candidates_for(_nz(desc)) if c != default]:
             jz.jz_set_tiling(g.h, kc)
             ms = _time_ms(torch, lambda: g.nsteps(1, cfl=cfl), stream, reps)
             if ms < best["ms"]:
@@ -85,9 +90,10 @@ def tune_grid(desc: dict, flow: dict, cfl: float = 0.5, reps: int = 3, device: i
 
 def tune_batch(cases: list[tuple[dict, dict]], cfl: float = 0.5, reps: int = 2, device: int = 0,
                candidates=(4, 8, 16, 32, 64, 0)) -> dict:
-    """Best tile shape and uniform k-chunk length (0 = whole k range) for a
-    batch of grids (list of (grid desc, flow)), timed with batched steps on
-    scratch grids: {"shape": (ti, tj) or None, "kc": planes, "ms": step time}."""
+    """Best tile shape and k-chunk length for a batch of grids (list of (grid
+    desc, flow)), timed with batched steps on scratch grids: {"shape": (ti, tj)
+    or None, "kc": planes of every grid (0 = whole k range) or CHOSEN, "ms": step
+    time}."""
     import torch
     sig = ("batch",) + tuple(sorted((d.get("precision", 0), d.get("geom", 0), d["ni"], d["nj"], d["nk"])
                                     for d, _ in cases))
@@ -97,7 +103,7 @@ def tune_batch(cases: list[tuple[dict, dict]], cfl: float = 0.5, reps: int = 2, 
     grids = [jz.Grid(d, stream=stream, device=device).init(f, 0) for d, f in cases]
     best = {"shape": None, "kc": None, "ms": float("inf")}
     for shape in _shapes(cases[0][0]):
-        for kc in candidates:
+        for kc in (CHOSEN, *candidates):  # CHOSEN first: no length is set yet
             for g in grids:
                 apply(g, {"shape": shape, "kc": kc})
             b = jz.Batch(grids, stream=stream)
@@ -112,5 +118,7 @@ def tune_batch(cases: list[tuple[dict, dict]], cfl: float = 0.5, reps: int = 2, 
 
 
 def apply_kc(grid: jz.Grid, kc: int) -> None:
+    if kc == CHOSEN:
+        return
     nz = _nz(grid.desc)
     jz.jz_set_tiling(grid.h, nz if kc == 0 else min(kc, nz))
