@@ -162,6 +162,27 @@ struct Consts {
   double muc, kpr, kprt;  // mu_inf (1 + S1), Cp / Pr, Cp / Pr_t
 };
 
+// Vreman's eddy viscosity (the formula of eddy_nu) from the gradients without
+// their factor J/2
+__device__ __forceinline__ double vreman_nu(const KConst<double>& c, const double g[4][3], double hJ, double J) {
+  double gj[3][3], b[3][3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+#pragma unroll
+    for (int m = 0; m < 3; ++m) gj[q][m] = mul(hJ, g[q][m]);
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int d = a; d < 3; ++d)
+      b[a][d] = fma(gj[a][2], gj[d][2], fma(gj[a][1], gj[d][1], mul(gj[a][0], gj[d][0])));
+  const double aa = add(add(b[0][0], b[1][1]), b[2][2]);
+  if (!(aa > 0.0)) return 0.0;
+  double B = fma(-b[0][1], b[0][1], mul(b[0][0], b[1][1]));
+  B = fma(-b[0][2], b[0][2], fma(b[0][0], b[2][2], B));
+  B = fma(-b[1][2], b[1][2], fma(b[1][1], b[2][2], B));
+  return mul(mul(mul(2.5, c.cs2), jm23_d(J)), __dsqrt_rn(__ddiv_rn(rmax(B, 0.0), aa)));
+}
+
 // A node before its directions: metrics, velocities, viscous flux vectors,
 // radii.  pm, pc, pp: primitive records (u, v, w, T, p) of the own column
 // below / at / above; P: the plane's primitive ring slot, o the node in it.
@@ -198,12 +219,7 @@ struct Node {
       if (ModelFlags<MD>::sgs(c)) {
         double nu_t;
         if (MD == kModelRuntime && c.vreman) {
-          double gj[4][3];
-#pragma unroll
-          for (int q = 0; q < 3; ++q)
-#pragma unroll
-            for (int m = 0; m < 3; ++m) gj[q][m] = mul(hJ, g[q][m]);
-          nu_t = eddy_nu<double, 1>(c, gj, J);
+          nu_t = vreman_nu(c, g, hJ, J);
         } else {  // Smagorinsky: (C_s Delta)^2 sqrt(2 S_ij S_ij), Delta^2 = J^(-2/3)
           const double dd = fma(g[2][2], g[2][2], fma(g[1][1], g[1][1], mul(g[0][0], g[0][0])));
           const double ss = fma(2.0, dd, fma(s12, s12, fma(s02, s02, mul(s01, s01))));
