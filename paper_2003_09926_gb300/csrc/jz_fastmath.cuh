@@ -123,5 +123,27 @@ __device__ __forceinline__ double jm23_d(double J) {
   return __hiloint2double(rhi, rlo);
 }
 
+// Five increments in FP64, exactly.  A conversion instruction runs on the FP64
+// pipe, which passes two lanes per cycle on a GB300 SM and which the five
+// additions and roundings of an update need too; for normal numbers the
+// exponent is re-biased with integer instructions instead (one check for all
+// five: separate ones cost what they saved).  160x128x128: 0.826 and 0.750 ms
+// per step.
+__device__ __forceinline__ void widen5(const float x[5], double y[5]) {
+  bool normal = true;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) normal = normal && (__float_as_uint(x[v]) & 0x7fffffffu) - 0x00800000u < 0x7f000000u;
+  if (normal) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const uint32_t b = __float_as_uint(x[v]);
+      y[v] = __hiloint2double((int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
+    }
+  } else {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) y[v] = (double)x[v];
+  }
+}
+
 }  // namespace stg
 }  // namespace jz

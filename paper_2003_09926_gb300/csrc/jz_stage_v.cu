@@ -484,28 +484,6 @@ __device__ __forceinline__ int role_of(int tid) {
 // every wait follows from the plane index.  On a bounded-wait timeout the
 // item records where it gave up, lets its copies in flight land and returns
 // false.
-// Five increments in FP64, exactly.  A conversion instruction runs on the FP64
-// pipe, which passes two lanes per cycle on a GB300 SM and which the five
-// additions and roundings of an update need too; for normal numbers the
-// exponent is re-biased with integer instructions instead (one check for all
-// five: separate ones cost what they saved).  160x128x128: 0.826 and 0.750 ms
-// per step.
-__device__ __forceinline__ void widen5(const float x[5], double y[5]) {
-  bool normal = true;
-#pragma unroll
-  for (int v = 0; v < 5; ++v) normal = normal && (__float_as_uint(x[v]) & 0x7fffffffu) - 0x00800000u < 0x7f000000u;
-  if (normal) {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      const uint32_t b = __float_as_uint(x[v]);
-      y[v] = __hiloint2double((int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
-    }
-  } else {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) y[v] = (double)x[v];
-  }
-}
-
 // S64: the state between time steps is FP64 (X.Q0d at the updated nodes): the
 // update adds the FP32 increment to it in FP64, stages 1-4 round their output
 // to FP32 (it feeds only the FP32 flux evaluation), and stage 5 writes both

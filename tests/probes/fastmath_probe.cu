@@ -15,6 +15,17 @@ __global__ void k_eval(int which, int n, const double* x, double* y) {
   }
 }
 
+// n groups of five FP32 values (as doubles) widened to FP64
+__global__ void k_widen(int n, const double* x, double* y) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  float f[5];
+  for (int v = 0; v < 5; ++v) f[v] = (float)x[5 * i + v];
+  double d[5];
+  widen5(f, d);
+  for (int v = 0; v < 5; ++v) y[5 * i + v] = d[v];
+}
+
 // y = f(x) for n host values; returns a CUDA error code
 extern "C" int fastmath_eval(int which, int n, const double* x, double* y) {
   double* d = nullptr;
@@ -22,7 +33,10 @@ extern "C" int fastmath_eval(int which, int n, const double* x, double* y) {
   if (e != cudaSuccess) return (int)e;
   e = cudaMemcpy(d, x, sizeof(double) * (size_t)n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    k_eval<<<(n + 255) / 256, 256>>>(which, n, d, d + n);
+    if (which == 4)
+      k_widen<<<(n / 5 + 255) / 256, 256>>>(n / 5, d, d + n);
+    else
+      k_eval<<<(n + 255) / 256, 256>>>(which, n, d, d + n);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpy(y, d + n, sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost);

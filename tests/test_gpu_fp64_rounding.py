@@ -1,6 +1,7 @@
 """Rounding errors of the FP64 kernels' building blocks, against extended
 precision: the elementary functions that they evaluate from the hardware's
-approximations, over mantissas and exponents, and the face flux."""
+approximations, over mantissas and exponents, the face flux, and the widening of
+the FP64-state update."""
 import ctypes as C
 import os
 import subprocess
@@ -10,7 +11,7 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
-RCP, SQRT, JM23, JM23_LIBRARY = range(4)
+RCP, SQRT, JM23, JM23_LIBRARY, WIDEN = range(5)
 
 
 P = C.POINTER(C.c_double)
@@ -154,3 +155,22 @@ def test_a_nan_sensor_reaches_the_face_flux(face):
     x[:, 24] = 1.5  # a density jump at the face
     assert face(n, 0.25, 2.0 ** -8, _dp(x), _dp(y)) == 0
     assert not np.isfinite(y[:2, 0]).any() and np.isfinite(y[2:]).all()
+
+
+def test_increments_are_widened_exactly(evaluate):
+    """Groups of five FP32 numbers of every exponent, zeros, subnormal numbers,
+    infinities and NaN among them: alone in a group, and in groups of their own."""
+    rng = np.random.default_rng(9)
+    x = rng.integers(0, 2 ** 32, 5 * 100_000, dtype=np.uint64).astype(np.uint32).view(np.float32)
+    special = np.array([0x0, 0x80000000, 0x1, 0x80000001, 0x7fffff, 0x807fffff, 0x800000, 0x80800000, 0x7f7fffff,
+                        0xff7fffff, 0x7f800000, 0xff800000, 0x7fc00000, 0xffc00000, 0x3f800000], np.uint32)
+    g = np.full((15, 5, 5), 1.25, np.float32)
+    for k in range(5):
+        g[:, k, k] = special.view(np.float32)
+    x = np.concatenate([x, special.view(np.float32), g.ravel()])
+    with np.errstate(invalid="ignore"):
+        want = x.astype(np.float64)
+    got = evaluate(WIDEN, want)
+    number = ~np.isnan(want)
+    np.testing.assert_array_equal(got[number].view(np.int64), want[number].view(np.int64))
+    assert np.isnan(got[~number]).all()
