@@ -145,8 +145,6 @@ __host__ __device__ __forceinline__ double unit53(uint64_t r) {
   return (double)(r >> 11) * (1.0 / 9007199254740992.0);
 }
 
-template <typename T> __device__ __forceinline__ T ld(const T* p) { return __ldg(p); }
-
 // Per-node diagnostic quantities of a conserved state q, in the state's
 // arithmetic type T: pressure and the squared Mach number (the maximum over
 // nodes is taken on the square; its root is taken once at the end).

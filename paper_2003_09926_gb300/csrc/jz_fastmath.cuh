@@ -10,8 +10,7 @@ namespace stg {
 
 // Elementary functions.  FP32 arithmetic uses the hardware approximations
 // (sqrt.approx, rcp.approx, ex2/lg2.approx: a few ulp, far below the FP32
-// error of the scheme itself); Fn<double> is the library's (boundary pass,
-// Vreman's model), the FP64 kernels' own functions follow it.
+// error of the scheme itself); the FP64 kernels' functions follow it.
 template <typename R> struct Fn;
 template <> struct Fn<float> {
   static __device__ __forceinline__ float sqrt_(float x) {
@@ -42,17 +41,6 @@ template <> struct Fn<float> {
     l *= -2.0f / 3.0f;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(l));
     return y;
-  }
-};
-template <> struct Fn<double> {
-  static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
-  static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-  static __device__ __forceinline__ double div(double a, double b) { return a / b; }
-  static __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-  static __device__ __forceinline__ double powp(double x, double e) { return pow(x, e); }
-  static __device__ __forceinline__ double jm23(double J) {
-    const double cb = cbrt(J);
-    return 1.0 / (cb * cb);
   }
 };
 

@@ -392,10 +392,13 @@ __device__ __forceinline__ bool node_value(const Layout& L, const double* inflow
     return true;
   }
   if (L.bc[f] == BC_AXIS) {  // azimuthal mean of the adjacent radial line
-    if (AXIS_IN) return false;
+    if constexpr (AXIS_IN) {
+      return false;
+    } else {
 #pragma unroll
-    for (int c = 0; c < 5; ++c) v[c] = (ST)axis[c * L.n[0] + mi];
-    return true;
+      for (int c = 0; c < 5; ++c) v[c] = (ST)axis[c * L.n[0] + mi];
+      return true;
+    }
   }
   // far field: nearest updated node, normal at the boundary node (on the
   // centreline the face metric vanishes: that of the adjacent radial node)
@@ -478,7 +481,7 @@ struct FillBlocks {
 // summed in azimuthal order in FP64 -- the sequential order the paper keeps
 // so that a partitioned run reproduces the serial one bit for bit.
 // A block takes 32 consecutive i of one variable (blockIdx.y); lane = i.
-// This is the general form, used for FP64 states: the loads are issued in
+// FP64 states: the loads are issued in
 // parallel, the azimuth going through shared memory in chunks of 24 KB (96
 // FP64 values per i), seven warps loading the next chunk (one coalesced row
 // of 32 i per load) while warp 0 adds the current one value by value in
@@ -488,15 +491,15 @@ constexpr int AX_BYTES = 24576;  // one chunk buffer; two are used
 
 // rows first + r, r = wr, wr + NW, ... < m, of the 32 i-columns into dst[r]:
 // all loads of a warp issued before the first store
-template <typename ST, int NW, int CH>
-__device__ __forceinline__ void ax_load(ST (*dst)[32], const ST* q, long long plane, int first, int m, int wr,
+template <int NW, int CH>
+__device__ __forceinline__ void ax_load(double (*dst)[32], const double* q, long long plane, int first, int m, int wr,
                                         bool live, int lane) {
   constexpr int U = (CH + NW - 1) / NW;
-  ST x[U];
+  double x[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int r = wr + u * NW;
-    x[u] = (live && r < m) ? q[(long long)(first + r) * plane] : ST(0);
+    x[u] = (live && r < m) ? q[(long long)(first + r) * plane] : 0.0;
   }
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -505,27 +508,25 @@ __device__ __forceinline__ void ax_load(ST (*dst)[32], const ST* q, long long pl
   }
 }
 
-template <typename ST>
-__device__ __forceinline__ void axis_mean(const Layout& L, const ST* __restrict__ Q, double* __restrict__ axis) {
-  constexpr int CH = AX_BYTES / (32 * (int)sizeof(ST));
-  __shared__ ST buf[2][CH][32];
+__device__ __forceinline__ void axis_mean(const Layout& L, const double* __restrict__ Q, double* __restrict__ axis) {
+  constexpr int CH = AX_BYTES / (32 * (int)sizeof(double));
+  __shared__ double buf[2][CH][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int v = blockIdx.y, P = L.pn[2], nch = (P + CH - 1) / CH;
   for (int bx = blockIdx.x; bx * 32 < L.n[0]; bx += gridDim.x) {  // block-uniform trip count
     const int i = bx * 32 + lane;
     const bool live = i < L.n[0];
-    const ST* q = Q + (long long)v * L.npad + L.at(live ? i : 0, 1, 0);
-    ax_load<ST, AX_WARPS, CH>(buf[0], q, L.plane, 0, min(CH, P), w, live, lane);  // chunk 0: every warp
+    const double* q = Q + (long long)v * L.npad + L.at(live ? i : 0, 1, 0);
+    ax_load<AX_WARPS, CH>(buf[0], q, L.plane, 0, min(CH, P), w, live, lane);  // chunk 0: every warp
     __syncthreads();
     double s = 0.0;
     for (int c = 0; c < nch; ++c) {
       const int base = c * CH, m = min(CH, P - base);
       if (w == 0) {
-        const ST* b = &buf[c & 1][0][lane];
-        for (int r = 0; r < m; ++r) s += (double)b[r * 32];
+        const double* b = &buf[c & 1][0][lane];
+        for (int r = 0; r < m; ++r) s += b[r * 32];
       } else if (c + 1 < nch) {
-        ax_load<ST, AX_WARPS - 1, CH>(buf[(c + 1) & 1], q, L.plane, base + CH, min(CH, P - base - CH), w - 1, live,
-                                      lane);
+        ax_load<AX_WARPS - 1, CH>(buf[(c + 1) & 1], q, L.plane, base + CH, min(CH, P - base - CH), w - 1, live, lane);
       }
       __syncthreads();
     }
@@ -633,7 +634,7 @@ __device__ __forceinline__ void axis_block(const Layout& L, float* Q, int ib, in
 // FP64 states: the means into the grid's axis table, before the boundary pass
 __global__ void __launch_bounds__(32 * AX_WARPS) k_axis_mean(const __grid_constant__ Layout L, const double* __restrict__ Q,
                                                              double* __restrict__ axis) {
-  axis_mean<double>(L, Q, axis);
+  axis_mean(L, Q, axis);
 }
 
 // threads of a boundary-pass block: small blocks spread the FP64 formulas over
@@ -697,7 +698,7 @@ __global__ void __launch_bounds__(32 * AX_WARPS)
 
 __global__ void __launch_bounds__(32 * AX_WARPS) k_axis_mean_batch(const BcCtx* __restrict__ ctx, int which) {
   const BcCtx& X = ctx[blockIdx.z];
-  if (X.L.cyl) axis_mean<double>(X.L, (const double*)X.Q[which], X.axis);
+  if (X.L.cyl) axis_mean(X.L, (const double*)X.Q[which], X.axis);
 }
 
 // Halo exchange between blocks of one grid (the paper's ghost exchange,

@@ -94,15 +94,15 @@ struct ModelFlags {
 //     b_ab = sum_m g[a][m] g[b][m] and B = b00 b11 - b01^2 + b00 b22 - b02^2
 //     + b11 b22 - b12^2 (the sum of b's principal 2x2 minors, >= 0; clamped at
 //     0 against rounding); 0 where all gradients vanish (g_am g_am = 0).
-//     B <= (g_am g_am)^2/3, so the model tends to 0 with the gradients.  In
-//     FP32 the reciprocal flushes subnormal operands to zero, so there the
-//     model is also taken as 0 where g_am g_am is below the smallest normal
-//     FP32 number; FP64 uses the plain > 0 test.
+//     B <= (g_am g_am)^2/3, so the model tends to 0 with the gradients.  The
+//     FP32 reciprocal flushes subnormal operands to zero, so the model is also
+//     taken as 0 where g_am g_am is below the smallest normal FP32 number (the
+//     FP64 kernel's own form uses the plain > 0 test).
 // EDDY: -1 the model of c (read at run time), 0 Smagorinsky, 1 Vreman.
 template <typename R, int EDDY = -1>
 __device__ __forceinline__ R eddy_nu(const KConst<R>& c, const R g[4][3], R Jn) {
   if (EDDY < 0 ? c.vreman != 0 : EDDY == 1) {
-    const R tiny = sizeof(R) == 4 ? R(1.17549435e-38f) : R(0);
+    const R tiny = R(1.17549435e-38f);
     R b[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)

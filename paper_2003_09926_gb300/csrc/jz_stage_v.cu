@@ -266,7 +266,7 @@ __device__ __forceinline__ void tm_free(unsigned char* smem) {
 // nu^k.  The node's own column comes in registers: primitive records of the
 // planes below / at / above (pm, pc, pp: u, v, w, T, p) and rho and e; its i
 // and j neighbours from the primitive ring slot sC of the plane.  DIR = 0:
-// all three directions; DIR = 1 / 2 / 3: direction i / j / k only.
+// all three directions; DIR = 1 / 2: direction i / j only.
 template <int DIR, int MD>
 __device__ __forceinline__ void node_v(const float4* __restrict__ PV, const float* __restrict__ PP,
                                        const float* __restrict__ met, int sC, const float pm5[5], const float pc5[5],
@@ -281,7 +281,7 @@ __device__ __forceinline__ void node_v(const float4* __restrict__ PV, const floa
   Jn = met[9 * MPL + mo];
   const float4* pc = PV + sC;
   const float u = pc5[0], v = pc5[1], w = pc5[2], T = pc5[3], p = pc5[4];
-  constexpr int K0 = DIR == 0 ? 0 : DIR - 1;  // DIR 3: direction k only
+  constexpr int K0 = DIR == 0 ? 0 : DIR - 1;
   constexpr int K1 = DIR == 0 ? 3 : DIR;
 
   float Fv[3][4];  // viscous flux vectors F_m (m = x, y, z), components 1..4
