@@ -64,7 +64,10 @@ extern "C" {
 #define JZ_GEOM_BOX 0      /* Cartesian box, optional tanh clustering and mapping */
 #define JZ_GEOM_CYLINDER 1 /* the paper's cylindrical jet grid (Section 3)        */
 
-/* precision modes: state/flux arithmetic, metric storage.  FP32 flux
+/* precision modes: state/flux arithmetic, metric storage.  The FP64 mode's
+ * reciprocals, square roots and J^(-2/3) are the kernels' own, no less precise
+ * than CUDA's (0.5 units in the last place, 1.2 for J^(-2/3); subnormal
+ * operands count as zero).  FP32 flux
  * arithmetic uses the hardware approximations of sqrt, reciprocal and
  * powers (a few ulp); so do the boundary formulas of JZ_P32 and JZ_P32_M64,
  * while JZ_P32_S64 evaluates them with IEEE FP32 operations.  JZ_P32 and
@@ -324,11 +327,12 @@ int jz_state_upload(jz_grid* g, const double* host, size_t n);
 
 /* Batched execution of many grids: per stage, one persistent launch whose
  * CTAs take (grid, tile, k-chunk) work items from a device queue, largest
- * first, plus one batched boundary fill (preceded by the centreline means
- * when a grid is cylindrical); per step one batched time-step reduction.  The batch borrows the grids (one precision mode, flow
- * parameters set; they must outlive the batch; a k-chunk length set with
- * jz_set_tiling is kept, the others are chosen for the whole batch) and a
- * caller-owned, 256-byte aligned device
+ * first, plus one batched boundary fill (it forms the centreline means of
+ * cylindrical FP32 grids; FP64 ones have them formed before it); per step one
+ * batched time-step reduction.  The batch borrows the grids (one precision
+ * mode, flow parameters set; they must outlive the batch; a k-chunk length set
+ * with jz_set_tiling is kept, the others are chosen for the whole batch; FP64
+ * grids all run 16 x 16 tiles) and a caller-owned, 256-byte aligned device
  * buffer of jz_batch_bytes bytes for its tables; work goes to `stream`
  * (the grids' own streams are not used, so order them against it).  Every
  * grid keeps its own CFL time step on the device, and its state is bitwise
@@ -418,10 +422,12 @@ int jz_profile_end(jz_grid* g);
 int jz_fma_peak(int fp64, double* tflops, void* stream);
 
 /* Tile shape of the fused stage kernel for this grid (for tuning and for
- * the batched tile table): ti x tj nodes per CTA, kc planes per CTA chunk.
- * jz_set_tiling may change kc (planes per chunk, >= 1); the (i, j) shape is
- * fixed per precision mode except for the FP32 vector-record kernel, whose
- * shape jz_set_tile_shape selects. */
+ * the batched tile table): ti x tj nodes per CTA, kc planes per CTA chunk, as
+ * the grid runs them when stepped alone (a batch may choose others).
+ * jz_set_tiling may change kc (planes per chunk, >= 1; more than the grid has
+ * are the whole column).  The (i, j) shape: jz_set_tile_shape selects it for
+ * the FP32 vector-record kernel; a JZ_P64 grid gets 16 x 16 or 8 x 8 with its
+ * default kc, by its size; the other modes have one each. */
 int jz_get_tiling(jz_grid* g, int* ti, int* tj, int* kc);
 int jz_set_tiling(jz_grid* g, int kc);
 
@@ -431,8 +437,8 @@ int jz_set_tiling(jz_grid* g, int kc);
  * per plane).  Both evaluate the same formulas; results agree to FP32
  * rounding.  Measured on the 256x192x192 mapped jet: 0.30 ms (2) and 0.55 ms
  * (0) per stage.  Grids of the other precision modes run one kernel only (the
- * scalar one for JZ_P64 and JZ_P32_M64, the vector-record one for
- * JZ_P32_S64): variant 0 is accepted there without effect; JZ_EINVAL for
+ * scalar one for JZ_P32_M64, the vector-record one for JZ_P32_S64, an FP64
+ * kernel of its own for JZ_P64): variant 0 is accepted there without effect; JZ_EINVAL for
  * variant 2 there, and for other variants.  A batch uses its first grid's variant. */
 int jz_set_stage_variant(jz_grid* g, int variant);
 

@@ -1007,11 +1007,14 @@ void bc_fill_items(const GridDev& g, int grid, std::vector<int4>& out) {
 
 template <typename ST, typename MT, bool FAST>
 static void launch_fill_batch(const BcCtx* X, const int4* items, int nitems, int which, bool cyl, cudaStream_t s) {
-  if (cyl && sizeof(ST) == 4)
-    k_bc_fill_batch<ST, MT, FAST, true><<<nitems, 32 * AX_WARPS, 0, s>>>(X, items, which);
-  else
-    k_bc_fill_batch<ST, MT, FAST, false><<<nitems, fill_threads<ST, false>(), 0, s>>>(X, items, which);
   count_launches(1);
+  if constexpr (sizeof(ST) == 4) {
+    if (cyl) {
+      k_bc_fill_batch<ST, MT, FAST, true><<<nitems, 32 * AX_WARPS, 0, s>>>(X, items, which);
+      return;
+    }
+  }
+  k_bc_fill_batch<ST, MT, FAST, false><<<nitems, fill_threads<ST, false>(), 0, s>>>(X, items, which);
 }
 
 // cyl: some grid of the batch is cylindrical

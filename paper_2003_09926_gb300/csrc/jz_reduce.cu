@@ -31,7 +31,7 @@ int red_grid(int per_sm) {
 }
 
 // reciprocal and square root of the reduction: IEEE in FP32 (bound by memory),
-// the short forms in FP64 (bound by the FP64 pipe)
+// the FP64 kernels' own in FP64 (bound by the FP64 pipe), as precise
 __device__ __forceinline__ float rd_rcp(float x) { return 1.f / x; }
 __device__ __forceinline__ double rd_rcp(double x) { return stg::rcp_d(x); }
 __device__ __forceinline__ float rd_sqrt(float x) { return sqrt(x); }

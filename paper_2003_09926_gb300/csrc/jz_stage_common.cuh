@@ -1,5 +1,5 @@
-// jz_stage_common.cuh -- pieces shared by the scalar and the vector-record
-// fused stage kernels: ring record layout, flow constants in the arithmetic
+// jz_stage_common.cuh -- pieces shared by the fused stage kernels (scalar
+// and vector-record FP32, FP64): ring record layout, flow constants in the arithmetic
 // type, elementary-function choices, TMA / mbarrier helpers (inline PTX), the
 // per-grid kernel context and the per-launch stage selection.
 #pragma once

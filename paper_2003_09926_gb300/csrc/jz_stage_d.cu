@@ -691,8 +691,10 @@ template <class C, int MD>
 cudaError_t configure() {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(k_stage_d<C, MD>, a, (int)C::BYTES);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_stage_d_batch<C, MD>, a, (int)C::BYTES);
+  if constexpr (C::TI == 16) {  // batches run 16 x 16 tiles
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stage_d_batch<C, MD>, a, (int)C::BYTES);
+  }
+  return e;
 }
 
 template <class C, int MD>
@@ -736,8 +738,11 @@ int stage_d_ctas_per_sm(StageTiling t) { return t.ti == Small::TI ? Small::MINB 
 //   8 x 8: only while all CTAs are resident together; a plane takes
 //     9.5 + 7 c for c CTAs per SM and 15.6 at least (one CTA's three warps
 //     wait for one another's results half of the time).
-// 48x32x32: 8 x 8 with chunks of 3 planes 93 us per stage (2: 99, 5: 108),
-// 16 x 16 with chunks of 2 115 us.  77x42x54: 262 and 250 us.
+// (Fitted before the reciprocals and square roots took another instruction or
+// two; both tiles are 5% slower since.)  Measured, us per stage: 48x32x32, 8 x 8
+// with chunks of 2 planes (chosen) 104, of 3 98, of 5 114, 16 x 16 with chunks of 2
+// 121; 77x42x54, 16 x 16 with chunks of 6 (chosen) 263, 8 x 8 277 at best;
+// 56x36x30, 8 x 8 with chunks of 4 (chosen) 120, 16 x 16 156.
 void stage_d_split(const Layout& L, StageTiling& t, int& kc) {
   const int nz = L.hi[2] - L.lo[2] + 1;
   const long long sms = device_sm_count();
