@@ -202,7 +202,9 @@ cudaError_t launch_dep(void (*kernel)(KA...), dim3 grid, int threads, size_t sme
   c.stream = s;
   c.attrs = at;
   c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, kernel, KA(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&c, kernel, KA(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // reported here: the next caller that asks must not see it
+  return e;
 }
 
 // launch accounting (defined in jz_api.cu)
